@@ -112,9 +112,11 @@ typedef struct krr_opts {
                              the tensor-core product its P.V form) from the tuning table
                              where it has an entry for the configuration (krr_autotune,
                              krr_tune_load); 0 (default): from the cost model           */
-    int    tc_vfold;      /* 1 (default): the tensor-core product with one right-hand side
-                             folds v into the exponent (2^(t + log2|v_j|), columns taken
-                             in two sign groups), so its epilogue loads no V; 0: FFMA    */
+    int    tc_vfold;      /* 1 (default): the tensor-core product of two different point
+                             sets with one right-hand side folds v into the exponent
+                             (2^(t + log2|v_j|), columns taken in two sign groups), so its
+                             epilogue loads no V; 0: FFMA.  (The square product of one
+                             point set evaluates each pair once and takes neither.)      */
     int    reserved[1];
     double strong_f;      /* 0 (default): the build selects anchors by pivoted QR (Algorithm 1
                              step 3 as Section 3 remarks); f > 1: by strong RRQR with bound
@@ -426,6 +428,8 @@ int krr_batch_solve_grouped(const krr_problem* probs, int nprob, int nrhs, doubl
  * opts.autotune = 1.  Keys read "form=F w=W r=R lg=L": product form F (0 FP32
  * expansion, 1 tensor cores, 2 exact differences), feature width W (tensor-core K,
  * else the kernel dimension), R right-hand sides per launch, L = floor(log2 n).
+ * (The tensor-core product with R = 1 splits one sequence of work evenly; its count is the
+ * height of its row blocks, in 256 points, or 128 with 128-wide features; up to 4.)
  * Entries hold the split count, the P.V form (1 = on tensor cores) and the time.
  * The table is process-wide and guarded by a lock.
  *

@@ -290,7 +290,8 @@ static int ensure_raw_points(krr_ctx* ctx) {
 // cores, when built) or 2 (FP32 on raw coordinate differences).
 int square_product(krr_ctx* ctx, const float* V, int nrhs, float* Q, int form) {
     if (form == 1 && ctx->FA)
-        return launch_kmvm_tc(ctx, ctx->FA, ctx->n, ctx->FB, ctx->n, ctx->d, (float)ctx->beta, V, nrhs, Q);
+        return launch_kmvm_tc(ctx, ctx->FA, ctx->n, ctx->FB, ctx->n, ctx->d, (float)ctx->beta, V, nrhs, Q, nullptr,
+                              nullptr, true);
     if (form == 2) {
         KRR_RET(ensure_raw_points(ctx));
         return launch_kmvm(ctx, ctx->Praw, ctx->n, ctx->Praw, ctx->n, ctx->d, (float)ctx->beta, V, nrhs,
@@ -494,7 +495,8 @@ int krr_kmvm(krr_ctx* ctx, const float* Xr, long long nr, const float* Xc, long 
         int herr = 0;
         KRR_RET(bufT(ctx, "tc_err", 1, &err));
         KRR_TRY_CUDA(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
-        KRR_RET(launch_kmvm_tc(ctx, FA, nr, FB, nc, d, (float)beta, V, nrhs, Q));
+        KRR_RET(launch_kmvm_tc(ctx, FA, nr, FB, nc, d, (float)beta, V, nrhs, Q, nullptr, nullptr,
+                               Xr == Xc && nr == nc));
         KRR_TRY_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
         KRR_TRY_CUDA(cudaStreamSynchronize(ctx->stream));
         if (herr) return fail(ctx, KRR_E_TIMEOUT, "tensor-core product: a bounded wait timed out");

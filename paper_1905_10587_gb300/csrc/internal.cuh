@@ -315,7 +315,11 @@ size_t tc_feature_bytes(long long n, int d);
 int launch_tc_features(krr_ctx* ctx, const float* P, long long n, int d, int role, unsigned char* out);
 int launch_kmvm_tc(krr_ctx* ctx, const unsigned char* FA, long long nr, const unsigned char* FB,
                    long long nc, int d, float beta, const float* V, int nrhs, float* Q,
-                   const double* V64 = nullptr, double* Q64 = nullptr);
+                   const double* V64 = nullptr, double* Q64 = nullptr, bool same = false);
+// sym_tc.cu: the square product with one right-hand side, each pair evaluated once
+bool sym_tc_fits(long long n);
+int launch_kmvm_sym(krr_ctx* ctx, const unsigned char* FA, const unsigned char* FB, long long n, int d,
+                    float beta, const float* V, float* Q, int* err);
 int launch_sketch_tc(krr_ctx* ctx, const unsigned char* FA, const unsigned char* FB, long long n, int d,
                      const void* Om, int l, int njc_alloc, float* Y, int ldy);
 int launch_omega_bf16_tiled(krr_ctx* ctx, unsigned long long seed, int l, long long n, int nab,

@@ -1,0 +1,90 @@
+"""The symmetric tensor-core product (one right-hand side, square, each pair evaluated once)
+against the FP64 oracle: tile and row-block edges, every feature width, every work split, and
+columns far from unit scale.
+
+Tolerances are those of the tensor-core product's other tests: 1e-5 of the column norm, and per
+entry 3e-5 of sum_j |K_ij v_j| (the expansion's rounding, see test_gpu_parity.py).
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle import krr_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(n, d, seed=5):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    X = rng.normal(size=(n, d)).astype(np.float32)
+    v = rng.normal(size=(n, 1)).astype(np.float32)
+    return X, v, 0.6 * float(np.sqrt(d)), 1e-2
+
+
+def _product(X, v, sigma, beta, **opts):
+    from paper_1905_10587_gb300.api import KRR
+    Xd, vd = torch.from_numpy(X).cuda(), torch.from_numpy(v).cuda()
+    ctx = KRR(precision=1, **opts)
+    return ctx.kmvm(Xd, Xd, vd[:, 0], sigma, beta).cpu().numpy().astype(np.float64)
+
+
+def _check(q, X, v, sigma, beta):
+    ref = O.kmvm(X, v.astype(np.float64), sigma, beta)[:, 0]
+    mag = O.kmvm(X, np.abs(v.astype(np.float64)), sigma, beta)[:, 0]
+    assert np.linalg.norm(q - ref) <= 1e-5 * np.linalg.norm(ref)
+    assert np.all(np.abs(q - ref) <= 3e-5 * mag)
+
+
+# 1, 127 and 257 are single tiles and units; 2049, 2303 .. 2305 straddle tiles, units and row blocks;
+# d = 1, 2, 5, 7, 9 use 1 to 4 K steps of 256-column units, d = 10, 12, 16 5 to 7 of 128-column ones
+@pytest.mark.parametrize("n,d", [(1, 4), (127, 3), (257, 11), (2048, 1), (2049, 2), (2303, 5), (2304, 7), (2305, 9), (2049, 10),
+                                 (2561, 12), (4100, 16), (9001, 8)])
+def test_symmetric_product_matches_the_oracle(n, d):
+    X, v, sigma, beta = _case(n, d)
+    q = _product(X, v, sigma, beta)
+    _check(q, X, v, sigma, beta)
+
+
+@pytest.mark.parametrize("d,width", [(4, 64), (11, 128)])
+@pytest.mark.parametrize("split", [1, 2, 3, 4])
+def test_every_row_block_height(d, width, split):
+    from paper_1905_10587_gb300 import api
+    n = 3333
+    X, v, sigma, beta = _case(n, d)
+    api.tune_clear()
+    try:
+        api.tune_set(f"form=1 w={width} r=1 lg=11", split)
+        q = _product(X, v, sigma, beta, autotune=1)
+    finally:
+        api.tune_clear()
+    _check(q, X, v, sigma, beta)
+
+
+@pytest.mark.parametrize("scale", [0.0, 1e-38, 1e-30, 1e30])
+def test_columns_far_from_unit_scale(scale):
+    X, v, sigma, beta = _case(2500, 3)
+    v = (v * np.float32(scale)).astype(np.float32)
+    q = _product(X, v, sigma, beta)
+    if scale == 0.0:
+        assert not np.any(q)
+    else:
+        _check(q, X, v, sigma, beta)
+
+
+def test_points_and_vector_at_odd_addresses():
+    # a vector that starts 4 bytes past a 16-byte boundary
+    from paper_1905_10587_gb300.api import KRR
+    X, v, sigma, beta = _case(2100, 6)
+    Xd = torch.from_numpy(X).cuda()
+    buf = torch.zeros(2101, device="cuda")
+    buf[1:] = torch.from_numpy(v[:, 0]).cuda()
+    q = KRR(precision=1).kmvm(Xd, Xd, buf[1:], sigma, beta).cpu().numpy().astype(np.float64)
+    _check(q, X, v, sigma, beta)
+
+
+def test_results_do_not_depend_on_timing():
+    X, v, sigma, beta = _case(5000, 8)
+    first = _product(X, v, sigma, beta)
+    for _ in range(3):
+        again = _product(X, v, sigma, beta)
+        assert np.array_equal(first, again)
