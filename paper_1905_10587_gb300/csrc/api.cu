@@ -315,14 +315,14 @@ static int build_common(krr_ctx* ctx, const float* X, long long n, int d, double
     KRR_RET(bufT(ctx, "P", (size_t)n * ctx->ps, &ctx->P));
     Phase ph(ctx, PH_PREP);
     KRR_RET(launch_mean(ctx, X, n, d, mu));
-    KRR_RET(launch_pack(ctx, X, n, d, mu, ctx->s, ctx->P));
     ctx->FA = ctx->FB = nullptr;
     ctx->Praw = nullptr;
     if (use_tc(ctx, d)) {
         KRR_RET(bufT(ctx, "tc_FA", tc_feature_bytes(n, d), &ctx->FA));
         KRR_RET(bufT(ctx, "tc_FB", tc_feature_bytes(n, d), &ctx->FB));
-        KRR_RET(launch_tc_features(ctx, ctx->P, n, d, 0, ctx->FA));
-        KRR_RET(launch_tc_features(ctx, ctx->P, n, d, 1, ctx->FB));
+        KRR_RET(launch_tc_pack(ctx, X, n, d, mu, ctx->s, ctx->P, ctx->FA, ctx->FB));
+    } else {
+        KRR_RET(launch_pack(ctx, X, n, d, mu, ctx->s, ctx->P));
     }
     return KRR_OK;
 }
@@ -465,8 +465,8 @@ int krr_kmvm(krr_ctx* ctx, const float* Xr, long long nr, const float* Xc, long 
     double* mu;
     float *Pc, *Pr;
     KRR_RET(bufT(ctx, "kmvm_mu", (size_t)d, &mu));
-    KRR_RET(bufT(ctx, "kmvm_Pc", (size_t)nc * ps, &Pc));
     if (raw) {
+        KRR_RET(bufT(ctx, "kmvm_Pc", (size_t)nc * ps, &Pc));
         // exact-difference form: raw coordinates (mu = 0, unit scale)
         KRR_TRY_CUDA(cudaMemsetAsync(mu, 0, sizeof(double) * d, ctx->stream));
         KRR_RET(launch_pack(ctx, Xc, nc, d, mu, 1.0, Pc));
@@ -478,32 +478,32 @@ int krr_kmvm(krr_ctx* ctx, const float* Xr, long long nr, const float* Xc, long 
         return launch_kmvm(ctx, Pr, nr, Pc, nc, d, (float)beta, V, nrhs, Q, (float)(-s));
     }
     KRR_RET(launch_mean(ctx, Xc, nc, d, mu));
-    KRR_RET(launch_pack(ctx, Xc, nc, d, mu, s, Pc));
-    if (Xr == Xc && nr == nc) {
-        Pr = Pc;
-    } else {
-        KRR_RET(bufT(ctx, "kmvm_Pr", (size_t)nr * ps, &Pr));
-        KRR_RET(launch_pack(ctx, Xr, nr, d, mu, s, Pr));
-    }
+    const bool same = Xr == Xc && nr == nc;
     if (use_tc(ctx, d)) {
         unsigned char *FA, *FB;
         KRR_RET(bufT(ctx, "kmvm_FA", tc_feature_bytes(nr, d), &FA));
         KRR_RET(bufT(ctx, "kmvm_FB", tc_feature_bytes(nc, d), &FB));
-        KRR_RET(launch_tc_features(ctx, Pr, nr, d, 0, FA));
-        KRR_RET(launch_tc_features(ctx, Pc, nc, d, 1, FB));
+        KRR_RET(launch_tc_pack(ctx, Xc, nc, d, mu, s, nullptr, same ? FA : nullptr, FB));
+        if (!same) KRR_RET(launch_tc_pack(ctx, Xr, nr, d, mu, s, nullptr, FA, nullptr));
         int* err;
         int herr = 0;
         KRR_RET(bufT(ctx, "tc_err", 1, &err));
         KRR_TRY_CUDA(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
         KRR_RET(launch_kmvm_tc(ctx, FA, nr, FB, nc, d, (float)beta, V, nrhs, Q, nullptr, nullptr,
-                               Xr == Xc && nr == nc));
+                               same));
         KRR_TRY_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
         KRR_TRY_CUDA(cudaStreamSynchronize(ctx->stream));
         if (herr) return fail(ctx, KRR_E_TIMEOUT, "tensor-core product: a bounded wait timed out");
         return KRR_OK;
     }
-    KRR_RET(launch_kmvm(ctx, Pr, nr, Pc, nc, d, (float)beta, V, nrhs, Q));
-    return KRR_OK;
+    KRR_RET(bufT(ctx, "kmvm_Pc", (size_t)nc * ps, &Pc));
+    KRR_RET(launch_pack(ctx, Xc, nc, d, mu, s, Pc));
+    Pr = Pc;
+    if (!same) {
+        KRR_RET(bufT(ctx, "kmvm_Pr", (size_t)nr * ps, &Pr));
+        KRR_RET(launch_pack(ctx, Xr, nr, d, mu, s, Pr));
+    }
+    return launch_kmvm(ctx, Pr, nr, Pc, nc, d, (float)beta, V, nrhs, Q);
 }
 
 int krr_residual_hp(krr_ctx* ctx, const float* X, long long n, int d, double sigma, double beta,

@@ -309,10 +309,11 @@ int square_product(krr_ctx* ctx, const float* V, int nrhs, float* Q, int form);
 // recurrence (squared norms compared).
 constexpr double kGapRestart2 = 4.0;
 
-// tc_kmvm.cu: BF16x3 tcgen05 product (d <= 16).  Features: role 0 rows, 1 columns.
+// tc_kmvm.cu: BF16x3 tcgen05 product (d <= 16).  Features: FA of rows, FB of columns.
 int tc_feature_kp(int d);
 size_t tc_feature_bytes(long long n, int d);
-int launch_tc_features(krr_ctx* ctx, const float* P, long long n, int d, int role, unsigned char* out);
+int launch_tc_pack(krr_ctx* ctx, const float* X, long long n, int d, const double* mu, double s, float* P,
+                   unsigned char* FA, unsigned char* FB);
 int launch_kmvm_tc(krr_ctx* ctx, const unsigned char* FA, long long nr, const unsigned char* FB,
                    long long nc, int d, float beta, const float* V, int nrhs, float* Q,
                    const double* V64 = nullptr, double* Q64 = nullptr, bool same = false);

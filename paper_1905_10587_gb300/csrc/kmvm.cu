@@ -24,69 +24,108 @@
 namespace krr {
 
 // ------------------------------------------------------------------ mean / pack
-__global__ void k_mean_partial(const float* __restrict__ X, long long n, int d,
-                               double* __restrict__ part) {
-    __shared__ double red[256];
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (int c = 0; c < d; ++c) {
-        double s = 0.0;
-        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-            s += (double)X[i * d + c];
-        red[threadIdx.x] = s;
+constexpr int MN_T = 256;
+
+// Sums the block's v (thread j holds a value of coordinate (t0 + j) mod d) by coordinate: after it
+// entry j < d of sm is the sum of coordinate (t0 + j) mod d.  The tree adds entries a multiple of
+// d apart, so that both belong to one coordinate.
+__device__ __forceinline__ void coord_sum(double v, int d, double* sm) {
+    sm[threadIdx.x] = v;
+    int m = d;
+    while (2 * m <= MN_T) m *= 2;                  // m = d 2^k <= MN_T < 2 m
+    __syncthreads();
+    if ((int)threadIdx.x + m < MN_T) sm[threadIdx.x] += sm[threadIdx.x + m];
+    for (m /= 2; m >= d; m /= 2) {
         __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) part[(size_t)blockIdx.x * d + c] = red[0];
-        __syncthreads();
+        if ((int)threadIdx.x < m) sm[threadIdx.x] += sm[threadIdx.x + m];
     }
+    __syncthreads();
 }
 
-__global__ void k_mean_final(const double* __restrict__ part, int nblk, int d, long long n,
-                             double* __restrict__ mu) {
-    int c = threadIdx.x;
-    if (c >= d) return;
+// Per-block sums of every coordinate.  The array is read flat and coalesced: a stride that is a
+// multiple of d keeps each thread on one coordinate.  (A pass per coordinate with strided loads
+// took 20 us at n = 10^5, d = 8, and a one-thread-per-coordinate final sum 29 us.)
+__global__ void __launch_bounds__(MN_T) k_mean_partial(const float* __restrict__ X, long long n, int d,
+                                                       double* __restrict__ part) {
+    __shared__ double sm[MN_T];
+    const long long t = (long long)blockIdx.x * MN_T + threadIdx.x;
+    const long long stride = (long long)gridDim.x * MN_T / d * d;
     double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += part[(size_t)b * d + c];
-    mu[c] = s / (double)n;
+    if (t < stride) {
+#pragma unroll 4
+        for (long long i = t; i < n * d; i += stride) s += (double)X[i];
+    }
+    coord_sum(s, d, sm);
+    const int c = (int)(t % d);
+    if (threadIdx.x < d) part[(size_t)blockIdx.x * d + c] = sm[threadIdx.x];
+}
+
+__global__ void __launch_bounds__(MN_T) k_mean_final(const double* __restrict__ part, int nblk, int d, long long n,
+                                                     double* __restrict__ mu) {
+    __shared__ double sm[MN_T];
+    const int stride = MN_T / d * d;
+    double s = 0.0;
+    if (threadIdx.x < stride) {
+#pragma unroll 4
+        for (int i = threadIdx.x; i < nblk * d; i += stride) s += part[i];
+    }
+    coord_sum(s, d, sm);
+    if (threadIdx.x < d) mu[threadIdx.x] = sm[threadIdx.x] / (double)n;
 }
 
 int launch_mean(krr_ctx* ctx, const float* X, long long n, int d, double* mu) {
     const int nblk = (int)std::min<long long>(2 * ctx->num_sms, ceil_div(n, 256));
     double* part;
     KRR_RET(bufT(ctx, "mean_part", (size_t)nblk * d, &part));
-    k_mean_partial<<<nblk, 256, 0, ctx->stream>>>(X, n, d, part);
+    k_mean_partial<<<nblk, MN_T, 0, ctx->stream>>>(X, n, d, part);
     KRR_CHECK_LAUNCH();
-    k_mean_final<<<1, 64, 0, ctx->stream>>>(part, nblk, d, n, mu);
+    k_mean_final<<<1, MN_T, 0, ctx->stream>>>(part, nblk, d, n, mu);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
 
-__global__ void k_pack(const float* __restrict__ X, long long n, int d, int dk, int ps,
-                       const double* __restrict__ mu, double sq, float* __restrict__ P) {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// One thread per point, its packed row in registers and stored as float4s (scalar stores of each
+// coordinate took 20 us at n = 10^5, d = 8).  DK is the kernel dimension; d <= DK.
+template <int DK>
+__global__ void __launch_bounds__(128) k_pack(const float* __restrict__ X, long long n, int d,
+                                              const double* __restrict__ mu, double sq, float* __restrict__ P) {
+    constexpr int PS = (DK + 1 + 3) / 4 * 4;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    float p[PS];
     double nrm = 0.0;
-    float* out = P + i * ps;
-    for (int c = 0; c < ps; ++c) {
-        float v = 0.f;
-        if (c < d) v = (float)(((double)X[i * d + c] - mu[c]) * sq);
-        if (c < dk) {
-            out[c] = v;
-            nrm += (double)v * (double)v;
-        } else {
-            out[c] = 0.f;
+#pragma unroll
+    for (int c = 0; c < PS; ++c) {
+        p[c] = 0.f;
+        if (c < DK && c < d) {
+            p[c] = (float)(((double)X[i * d + c] - mu[c]) * sq);
+            nrm += (double)p[c] * (double)p[c];
         }
     }
-    out[dk] = (float)(-nrm);
+    p[DK] = (float)(-nrm);
+#pragma unroll
+    for (int c = 0; c < PS; c += 4)
+        reinterpret_cast<float4*>(P + i * PS)[c / 4] = make_float4(p[c], p[c + 1], p[c + 2], p[c + 3]);
+}
+
+static bool pack_on(cudaStream_t stream, const float* X, long long n, int d, const double* mu, double sq,
+                    float* P) {
+    const unsigned grid = ceil_div(n, 128);
+    switch (kernel_dim(d)) {
+#define KRR_D(v) \
+    case v: k_pack<v><<<grid, 128, 0, stream>>>(X, n, d, mu, sq, P); return true;
+        KRR_D(1) KRR_D(2) KRR_D(3) KRR_D(4) KRR_D(5) KRR_D(6) KRR_D(7) KRR_D(8)
+        KRR_D(9) KRR_D(10) KRR_D(11) KRR_D(12) KRR_D(13) KRR_D(14) KRR_D(15) KRR_D(16)
+        KRR_D(24) KRR_D(32) KRR_D(48) KRR_D(64)
+#undef KRR_D
+    }
+    return false;
 }
 
 int launch_pack(krr_ctx* ctx, const float* X, long long n, int d, const double* mu, double s,
                 float* P) {
-    const int dk = kernel_dim(d);
-    const int ps = packed_stride(d);
-    k_pack<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(X, n, d, dk, ps, mu, std::sqrt(s), P);
+    if (!pack_on(ctx->stream, X, n, d, mu, std::sqrt(s), P))
+        return fail(ctx, KRR_E_INVAL, "pack: unsupported dimension");
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -820,10 +859,10 @@ int kmvm_into_scratch(cudaStream_t stream, int num_sms, const float* Xr, long lo
     float* Pr = same ? Pc : reinterpret_cast<float*>(scratch + off_pr);
     double* part = reinterpret_cast<double*>(scratch + off_part);
     const double s = 1.4426950408889634 / (2.0 * sigma * sigma);
-    k_mean_partial<<<nblk_mean, 256, 0, stream>>>(Xc, nc, d, mpart);
-    k_mean_final<<<1, 64, 0, stream>>>(mpart, nblk_mean, d, nc, mu);
-    k_pack<<<ceil_div(nc, 256), 256, 0, stream>>>(Xc, nc, d, dk, ps, mu, std::sqrt(s), Pc);
-    if (!same) k_pack<<<ceil_div(nr, 256), 256, 0, stream>>>(Xr, nr, d, dk, ps, mu, std::sqrt(s), Pr);
+    k_mean_partial<<<nblk_mean, MN_T, 0, stream>>>(Xc, nc, d, mpart);
+    k_mean_final<<<1, MN_T, 0, stream>>>(mpart, nblk_mean, d, nc, mu);
+    pack_on(stream, Xc, nc, d, mu, std::sqrt(s), Pc);
+    if (!same) pack_on(stream, Xr, nr, d, mu, std::sqrt(s), Pr);
     for (int done = 0; done < nrhs;) {
         const int left = nrhs - done;
         const int chunk = left >= 16 ? 16 : left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;

@@ -19,6 +19,7 @@
 #include "tc_ptx.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <string>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -125,48 +126,84 @@ __device__ __forceinline__ void split3(float v, __nv_bfloat16& h, __nv_bfloat16&
     l = __float2bfloat16_rn(r2);
 }
 
-// Features of point i (packed xh, a at P[i*ps + dk]) written into 128-row tiles in the
-// 128-byte swizzled layout (K slabs of 64): role 0 = row operand, role 1 = column
-// operand.  The row operand also has ones at K = 6 dk + 6 .. 6 dk + 8 (see the V-folded
-// product).  Rows beyond n and the remaining K columns are zero.
-__global__ void k_tc_features(const float* __restrict__ P, long long n, int dk, int ps, int Kp,
-                              int role, long long nrows_pad, unsigned char* __restrict__ out) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nrows_pad) return;
-    const long long tile = i >> 7;
-    const int r = (int)(i & 127);
-    unsigned char* base = out + tile * (128LL * Kp * 2);
-    const __nv_bfloat16 one = __float2bfloat16_rn(1.f), zero = __float2bfloat16_rn(0.f);
-    auto put = [&](int k, __nv_bfloat16 v) {
-        *reinterpret_cast<__nv_bfloat16*>(base + tile_off_sw(r, k, 128)) = v;
-    };
-    if (i >= n) {
-        for (int k = 0; k < Kp; ++k) put(k, zero);
-        return;
-    }
-    int k = 0;
-    for (int c = 0; c < dk; ++c) {
-        const float x = P[i * ps + c];
-        __nv_bfloat16 h, m, l;
-        if (role == 0) {
-            split3(2.f * x, h, m, l);
-            put(k++, h); put(k++, h); put(k++, m); put(k++, h); put(k++, m); put(k++, l);
-        } else {
-            split3(x, h, m, l);
-            put(k++, h); put(k++, m); put(k++, h); put(k++, l); put(k++, m); put(k++, h);
+// Packs 128 points (one feature tile) and builds their features: xh = (x - mu) sqrt(s) and
+// a = -||xh||^2 as k_pack has them, into P (unless null) and into the tiles of the row operand FA
+// and the column operand FB (unless null): 128 rows in the 128-byte swizzled layout (K slabs of
+// 64).  The row operand also has ones at K = 6 D + 6 .. 6 D + 8 (see the V-folded product).
+// Points beyond n and the remaining K columns are zero.
+// A tile is built in shared memory, where a thread writes its point's row in 16-byte chunks, and
+// leaves as one contiguous copy: storing the 64 values of a row two bytes at a time from each
+// thread took 61 us per operand at n = 10^5, d = 8.
+template <int D>
+__global__ void __launch_bounds__(128)
+k_tc_pack(const float* __restrict__ X, long long n, int d, const double* __restrict__ mu, double sq,
+          float* __restrict__ P, unsigned char* __restrict__ FA, unsigned char* __restrict__ FB) {
+    constexpr int PS = (D + 1 + 3) / 4 * 4, KP = ((6 * D + 6) + 63) / 64 * 64;
+    __shared__ __align__(16) uint4 tile[128 * KP / 8];
+    const int r = threadIdx.x;
+    const long long i = (long long)blockIdx.x * 128 + r;
+    const bool ok = i < n;
+    float p[PS];
+    double nrm = 0.0;
+#pragma unroll
+    for (int c = 0; c < PS; ++c) {
+        p[c] = 0.f;
+        if (c < D && ok) {
+            p[c] = (float)(((double)X[i * d + c] - mu[c]) * sq);
+            nrm += (double)p[c] * (double)p[c];
         }
     }
-    __nv_bfloat16 a1, a2, a3;
-    split3(P[i * ps + dk], a1, a2, a3);
-    if (role == 0) {
-        put(k++, a1); put(k++, a2); put(k++, a3); put(k++, one); put(k++, one); put(k++, one);
-        // three more ones, against the column operand's log2|v_j| in the V-folded product
-        // (zero in the plain column features, so they add nothing elsewhere)
-        put(k++, one); put(k++, one); put(k++, one);
-    } else {
-        put(k++, one); put(k++, one); put(k++, one); put(k++, a1); put(k++, a2); put(k++, a3);
+    p[D] = (float)(-nrm);
+    if (P && ok) {
+#pragma unroll
+        for (int c = 0; c < PS; c += 4)
+            reinterpret_cast<float4*>(P + i * PS)[c / 4] = make_float4(p[c], p[c + 1], p[c + 2], p[c + 3]);
     }
-    for (; k < Kp; ++k) put(k, zero);
+#pragma unroll
+    for (int role = 0; role < 2; ++role) {
+        unsigned char* out = role == 0 ? FA : FB;
+        if (!out) continue;                        // uniform
+        __nv_bfloat16 f[KP];
+        const __nv_bfloat16 one = __float2bfloat16_rn(ok ? 1.f : 0.f);
+#pragma unroll
+        for (int k = 0; k < KP; ++k) f[k] = __float2bfloat16_rn(0.f);
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            __nv_bfloat16 h, m, l;
+            __nv_bfloat16* o = f + 6 * c;
+            if (role == 0) {
+                split3(2.f * p[c], h, m, l);
+                o[0] = h; o[1] = h; o[2] = m; o[3] = h; o[4] = m; o[5] = l;
+            } else {
+                split3(p[c], h, m, l);
+                o[0] = h; o[1] = m; o[2] = h; o[3] = l; o[4] = m; o[5] = h;
+            }
+        }
+        __nv_bfloat16 a[3];
+        split3(p[D], a[0], a[1], a[2]);
+#pragma unroll
+        for (int w = 0; w < 3; ++w) {
+            f[6 * D + w] = role == 0 ? a[w] : one;
+            f[6 * D + 3 + w] = role == 0 ? one : a[w];
+            // against the column operand's log2|v_j| in the V-folded product (zero in the plain
+            // column features, so they add nothing elsewhere)
+            if (role == 0 && 6 * D + 6 + w < KP) f[6 * D + 6 + w] = one;
+        }
+        __syncthreads();                           // the tile before has left
+#pragma unroll
+        for (int ch = 0; ch < KP / 8; ++ch) {
+            uint32_t w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                w[u] = (uint32_t)__bfloat16_as_ushort(f[8 * ch + 2 * u]) |
+                       ((uint32_t)__bfloat16_as_ushort(f[8 * ch + 2 * u + 1]) << 16);
+            tile[tile_off_sw(r, 8 * ch, 128) / 16] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        __syncthreads();
+        uint4* dst = reinterpret_cast<uint4*>(out + (size_t)blockIdx.x * (128 * KP * 2));
+#pragma unroll
+        for (int e = 0; e < KP / 8; ++e) dst[e * 128 + r] = tile[e * 128 + r];
+    }
 }
 
 // ------------------------------------------------------------------ V folded into the exponent
@@ -1258,12 +1295,19 @@ int launch_sketch_tc(krr_ctx* ctx, const unsigned char* FA, const unsigned char*
     return KRR_OK;
 }
 
-int launch_tc_features(krr_ctx* ctx, const float* P, long long n, int d, int role,
-                       unsigned char* out) {
-    const int dk = kernel_dim(d), Kp = tc_feature_kp(d);
-    const long long npad = (n + 255) / 256 * 256;
-    k_tc_features<<<ceil_div(npad, 256), 256, 0, ctx->stream>>>(P, n, dk, packed_stride(d), Kp, role,
-                                                                npad, out);
+// Packed points (P may be null) and features (FA, FB may be null) of X; see k_tc_pack.
+int launch_tc_pack(krr_ctx* ctx, const float* X, long long n, int d, const double* mu, double s, float* P,
+                   unsigned char* FA, unsigned char* FB) {
+    const unsigned grid = (unsigned)((n + 255) / 256 * 2);   // whole 256-point units
+    const double sq = std::sqrt(s);
+    switch (kernel_dim(d)) {
+#define KRR_D(v) \
+    case v: k_tc_pack<v><<<grid, 128, 0, ctx->stream>>>(X, n, d, mu, sq, P, FA, FB); break;
+        KRR_D(1) KRR_D(2) KRR_D(3) KRR_D(4) KRR_D(5) KRR_D(6) KRR_D(7) KRR_D(8)
+        KRR_D(9) KRR_D(10) KRR_D(11) KRR_D(12) KRR_D(13) KRR_D(14) KRR_D(15) KRR_D(16)
+#undef KRR_D
+        default: return fail(ctx, KRR_E_INVAL, "tensor-core features need d <= 16");
+    }
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
