@@ -267,6 +267,11 @@ int launch_kmvm_reduce(krr_ctx* ctx, const double* part, int splits, int nr, int
 int launch_kmvm_dsigma(krr_ctx* ctx, const float* Pr, long long nr, const float* Pc, long long nc,
                        int d, const float* V, float* Q);
 
+// sym_f32.cu: the square product with one right-hand side, each pair evaluated once
+bool sym_f32_fits(long long n, int d);
+int launch_kmvm_sym_f32(krr_ctx* ctx, const float* P, long long n, int d, float beta, const float* V, float* Q,
+                        float raw_nsc);
+
 // tune.cu: tuned work splits.  Key of a product configuration; the table entry for it
 // (only with opts.autotune and outside tuning); the split count to use (forced, tuned or
 // the cost model's `analytic`, clamped to [1, ntiles]; also recorded in ctx->last_splits).

@@ -642,6 +642,8 @@ static int choose_splits(int nblk, int ntiles, int slots) {
     return best;
 }
 
+int kernel_occupancy(const void* fn, int threads) { return occupancy(nullptr, fn, threads); }
+
 int choose_splits_public(int nblk, int ntiles, int slots) { return choose_splits(nblk, ntiles, slots); }
 
 int launch_kmvm_reduce64(krr_ctx* ctx, const double* part, int nparts, int nr, int nrhs2,
@@ -664,6 +666,18 @@ int launch_kmvm(krr_ctx* ctx, const float* Pr, long long nr, const float* Pc, lo
         const int left = nrhs - done;
         const int chunk = comp ? (left >= 4 ? 4 : 2)
                                : left >= 16 ? 16 : left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
+        // one right-hand side, one point set: each pair once (see sym_f32.cu)
+        if (chunk == 1 && !hp && Pr == Pc && nr == nc && sym_f32_fits(nr, d)) {
+            const int rc = launch_kmvm_sym_f32(ctx, Pr, nr, d, beta, V + (size_t)done * nc, Q + (size_t)done * nr,
+                                               raw_nsc);
+            ctx->last_splits = 1;
+            if (rc == KRR_OK) {
+                done += chunk;
+                continue;
+            }
+            if (rc != KRR_E_NOMEM) return rc;   // no room for its partial sums: the form below
+            ctx->err.clear();
+        }
         int R = 4;
         kmvm_fn fn = comp ? pick_comp(dk, chunk, &R) : pick(dk, chunk, &R, raw);
         if (!fn) return fail(ctx, KRR_E_INVAL, "kmvm: unsupported dimension");

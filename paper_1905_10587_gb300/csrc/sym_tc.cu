@@ -35,6 +35,7 @@
 // tiles 10% slower.  Fetching v a tile ahead and asking for the next tile's barrier a step ahead
 // gave 5% together, folding row and column sums under the next tile's exponentials 4%.
 #include "internal.cuh"
+#include "sym.cuh"
 #include "tc_ptx.cuh"
 
 #include <algorithm>
@@ -44,7 +45,6 @@ namespace krr {
 
 constexpr int SY_EW = 8;                         // epilogue warps: 2 column halves x 4 lane quarters
 constexpr int SY_THREADS = 32 * (2 + SY_EW);
-constexpr int SY_T = 128;                        // rows per tile
 constexpr int SY_RTMAX = 8;                      // most row tiles per block
 // buffers of the quarters' column sums, by column unit width (see column_done)
 constexpr int sy_nc(int BN) { return BN == 256 ? 3 : 4; }
@@ -56,65 +56,8 @@ struct SyShared {
     int abort;
 };
 
-// The points in column units of BN and row blocks of RU units (RU * BN / 128 row tiles).  Row
-// block I has the units I * RU .. NU - 1; first(I) (block, unit) pairs come before its own.
-struct SyGrid {
-    int n, BN, NU, RU, nblk, G;
-    long long W;                                  // (block, unit) pairs in all
-    __host__ __device__ int row_tiles(int I) const { return min(RU, NU - I * RU) * (BN / SY_T); }
-    __host__ __device__ int rows() const { return RU * BN; }
-    __host__ __device__ long long first(int I) const {
-        return (long long)I * NU - (long long)RU * ((long long)I * (I - 1) / 2);
-    }
-    // the row block of pair u
-    __host__ __device__ int block_of(long long u) const {
-        int lo = 0, hi = nblk - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (first(mid) <= u) lo = mid;
-            else hi = mid - 1;
-        }
-        return lo;
-    }
-    __host__ __device__ long long run_begin(int s) const { return W * s / G; }
-    // the run that holds pair u: the largest s with run_begin(s) <= u
-    __host__ __device__ int run_of(long long u) const { return (int)(((u + 1) * G - 1) / W); }
-    // first entry of column unit T's slots (T / RU of them, BN entries each)
-    __host__ __device__ long long col_base(int T) const {
-        const long long b = T / RU, r = T % RU;
-        return BN * (RU * (b * (b - 1) / 2) + r * b);
-    }
-    static __host__ __device__ int min(int a, int b) { return a < b ? a : b; }
-};
-
-__device__ __forceinline__ unsigned long long sy_pack(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void sy_unpack(unsigned long long v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ void sy_fma(unsigned long long& d, unsigned long long a, unsigned long long b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
 __device__ __forceinline__ void sy_bar(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
-// Sums each a[m] over the lanes that differ in bit ST and the lower bits halved in turn, down to
-// N >> levels values: a lane keeps the half of the values its bit selects and sends the other.
-template <int N, int ST>
-__device__ __forceinline__ void lane_sum(float* a, int lane) {
-    constexpr int H = N / 2;
-    const bool up = (lane & ST) != 0;
-#pragma unroll
-    for (int m = 0; m < H; ++m) {
-        const float send = up ? a[m] : a[m + H];
-        const float keep = up ? a[m + H] : a[m];
-        a[m] = keep + __shfl_xor_sync(0xffffffffu, send, ST);
-    }
-    if constexpr (ST == 16 || ST == 8 || ST == 2) lane_sum<H, ST / 2>(a, lane);
 }
 
 // v zero-padded to whole tiles (16-byte aligned bulk copies; padding columns add nothing), and
@@ -519,7 +462,7 @@ k_kmvm_sym(const unsigned char* __restrict__ FA, const unsigned char* __restrict
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// q_i = ksc vscale (sum of point i's column and row slots) + beta v_i.  One block per tile: 128 points
+// q_i = ksc vscale (sum of point i's column and row slots) + beta v_i (vscale null: 1).  One block per tile: 128 points
 // x 4 interleaved groups of column slots.
 constexpr int SYR_G = 4;
 __global__ void __launch_bounds__(SY_T * SYR_G)
@@ -550,8 +493,15 @@ k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __rest
         double t = red[0][x];
 #pragma unroll
         for (int w = 1; w < SYR_G; ++w) t += red[w][x];
-        Q[i] = (float)(t * (ksc * *vscale) + (beta != 0.f ? (double)beta * V[i] : 0.0));
+        Q[i] = (float)(t * (vscale ? ksc * *vscale : ksc) + (beta != 0.f ? (double)beta * V[i] : 0.0));
     }
+}
+
+int launch_sym_reduce(krr_ctx* ctx, const SyGrid& g, const float2* rowpart, const float2* colpart, const float* V,
+                      float beta, double ksc, const double* vscale, float* Q) {
+    k_sym_reduce<<<g.NU * g.BN / SY_T, SY_T * SYR_G, 0, ctx->stream>>>(g, rowpart, colpart, V, beta, ksc, vscale, Q);
+    KRR_CHECK_LAUNCH();
+    return KRR_OK;
 }
 
 static size_t sym_smem(int Kp, int BN, int RU) {
@@ -635,10 +585,7 @@ int launch_kmvm_sym(krr_ctx* ctx, const unsigned char* FA, const unsigned char* 
     fn<<<g.G, SY_THREADS, smem, ctx->stream>>>(FA, FB, Kp, g, Vp, rowpart, colpart, bmax, nbmax, vscale, err,
                                                wlimit, ctx->opts.test_stall_copies);
     KRR_CHECK_LAUNCH();
-    k_sym_reduce<<<np / SY_T, SY_T * SYR_G, 0, ctx->stream>>>(g, rowpart, colpart, V, beta, ex2_bias_scale(ctx), vscale,
-                                                                 Q);
-    KRR_CHECK_LAUNCH();
-    return KRR_OK;
+    return launch_sym_reduce(ctx, g, rowpart, colpart, V, beta, ex2_bias_scale(ctx), vscale, Q);
 }
 
 }  // namespace krr

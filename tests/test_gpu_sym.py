@@ -1,8 +1,8 @@
-"""The symmetric tensor-core product (one right-hand side, square, each pair evaluated once)
-against the FP64 oracle: tile and row-block edges, every feature width, every work split, and
+"""The symmetric products (one right-hand side, square, each pair evaluated once) against the
+FP64 oracle: tile and row-block edges, every feature width, every work split, and
 columns far from unit scale.
 
-Tolerances are those of the tensor-core product's other tests: 1e-5 of the column norm, and per
+Tolerances are those of the products' other tests: 1e-5 of the column norm, and per
 entry 3e-5 of sum_j |K_ij v_j| (the expansion's rounding, see test_gpu_parity.py).
 """
 import numpy as np
@@ -21,10 +21,10 @@ def _case(n, d, seed=5):
     return X, v, 0.6 * float(np.sqrt(d)), 1e-2
 
 
-def _product(X, v, sigma, beta, **opts):
+def _product(X, v, sigma, beta, precision=1, **opts):
     from paper_1905_10587_gb300.api import KRR
     Xd, vd = torch.from_numpy(X).cuda(), torch.from_numpy(v).cuda()
-    ctx = KRR(precision=1, **opts)
+    ctx = KRR(precision=precision, **opts)
     return ctx.kmvm(Xd, Xd, vd[:, 0], sigma, beta).cpu().numpy().astype(np.float64)
 
 
@@ -43,6 +43,25 @@ def test_symmetric_product_matches_the_oracle(n, d):
     X, v, sigma, beta = _case(n, d)
     q = _product(X, v, sigma, beta)
     _check(q, X, v, sigma, beta)
+
+
+# FP32 forms: 128-column tiles, 256-row blocks; four rows per thread for differences above d = 10,
+# an odd number of staged values per column (d odd or even by form), d = 4, 8, 12, 16 with a packed
+# row that ends in the norm or spills into the next float4
+@pytest.mark.parametrize("precision", [0, 2])
+@pytest.mark.parametrize("n,d", [(1, 3), (127, 1), (128, 4), (129, 8), (255, 2), (257, 11), (1000, 7), (2305, 10),
+                                 (4099, 12), (3000, 16), (9001, 3)])
+def test_symmetric_fp32_products_match_the_oracle(n, d, precision):
+    X, v, sigma, beta = _case(n, d)
+    _check(_product(X, v, sigma, beta, precision=precision), X, v, sigma, beta)
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+def test_fp32_results_do_not_depend_on_timing(precision):
+    X, v, sigma, beta = _case(5000, 8)
+    first = _product(X, v, sigma, beta, precision=precision)
+    for _ in range(3):
+        assert np.array_equal(first, _product(X, v, sigma, beta, precision=precision))
 
 
 @pytest.mark.parametrize("d,width", [(4, 64), (11, 128)])
