@@ -107,3 +107,22 @@ def test_results_do_not_depend_on_timing():
     for _ in range(3):
         again = _product(X, v, sigma, beta)
         assert np.array_equal(first, again)
+
+
+# the float-float residual with one column: units of 64 x 64, 128 x 128 and 256 x 128 pairs (taken as
+# n grows), their edges, and odd and even strides of the staged points; bar as in test_gpu_parity.py
+@pytest.mark.parametrize("n,d", [(1, 2), (63, 1), (64, 8), (65, 16), (129, 5), (257, 4), (1000, 16), (3001, 3),
+                                 (7000, 2), (13001, 1)])
+def test_symmetric_residual(n, d):
+    from paper_1905_10587_gb300.api import KRR
+    rng = np.random.Generator(np.random.PCG64(31 * d + n))
+    X = (rng.normal(size=(n, d)) * 2 + 5).astype(np.float32)
+    A = rng.normal(size=(n, 1)) * 100
+    Y = rng.normal(size=(n, 1)).astype(np.float32)
+    sigma, beta = 0.4 * float(np.sqrt(d)), 1e-3
+    R = KRR().residual_hp(torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), torch.from_numpy(A).cuda(), sigma,
+                          beta, mode="ff").cpu().numpy()
+    rows = rng.choice(n, min(n, 1500), replace=False)
+    ref = Y[rows].astype(np.float64) - O.kmvm(X, A, sigma, 0.0, rows=rows) - beta * A[rows]
+    cond = O.kmvm(X, np.abs(A), sigma, 0.0, rows=rows) + beta * np.abs(A[rows]) + np.abs(Y[rows])
+    assert np.all(np.abs(R[rows] - ref) <= 2e-11 * cond)
