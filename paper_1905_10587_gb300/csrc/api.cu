@@ -97,7 +97,7 @@ int launch_cg_start(krr_ctx* ctx, const float* r, const float* z, int nrhs, doub
 int launch_cg_alpha(krr_ctx* ctx, const float* p, const float* q, int nrhs, double* part);
 int launch_cg_update_xr(krr_ctx* ctx, float* x, float* r, const float* p, const float* q, int nrhs,
                         double* part, double tol2);
-int launch_cg_beta_p(krr_ctx* ctx, float* p, const float* z, int nrhs, const double* rz_part);
+int launch_cg_beta_p(krr_ctx* ctx, float* p, const float* z, int nrhs, const double* rz_part, bool with_beta);
 int launch_cg_set_active(krr_ctx* ctx, const int* act_host, int nrhs);
 int launch_identity_apply(krr_ctx* ctx, const float* R, int nrhs, float* Z, double* rz_part);
 int launch_identity_apply64(krr_ctx* ctx, const double* R, int nrhs, double* Z, double* rz_part);
@@ -385,9 +385,12 @@ int krr_create(krr_ctx** out, const krr_opts* opts, void* stream) {
         return KRR_E_CUDA;
     }
     if (cudaMalloc(&ctx->cg, sizeof(CGScalars)) != cudaSuccess ||
-        cudaMallocHost(&ctx->cg_host, sizeof(CGScalars)) != cudaSuccess) {
+        cudaMallocHost(&ctx->cg_host, sizeof(CGScalars)) != cudaSuccess ||
+        cudaMemsetAsync(ctx->cg, 0, sizeof(CGScalars), ctx->stream) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->cg_read, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         if (ctx->cg) cudaFree(ctx->cg);
+        if (ctx->cg_host) cudaFreeHost(ctx->cg_host);
         delete ctx;
         return KRR_E_NOMEM;
     }
@@ -407,6 +410,7 @@ void krr_destroy(krr_ctx* ctx) {
         if (kv.second.p) cudaFree(kv.second.p);
     if (ctx->cg) cudaFree(ctx->cg);
     if (ctx->cg_host) cudaFreeHost(ctx->cg_host);
+    if (ctx->cg_read) cudaEventDestroy(ctx->cg_read);
     delete ctx;
 }
 
@@ -934,6 +938,16 @@ int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol
         double best = 1.0;
         std::vector<double> rec(nrhs);
         bool lanczos_on = true;
+        // z = M^-1 r of the recursive residual, and the b that comes with it (rz itself changes
+        // with p, so that a replaced residual can be applied again)
+        auto apply = [&]() -> int {
+            Phase ph(ctx, PH_APPLY);
+            if (ctx->opts.no_precond)
+                return hp ? launch_identity_apply64(ctx, rr64, nrhs, z64, part3)
+                          : launch_identity_apply(ctx, r, nrhs, z, part3);
+            if (hp) return launch_apply_precond64(ctx, rr64, nrhs, z64, part3);
+            return launch_apply_precond(ctx, r, nrhs, z, part3, true);
+        };
         while (true) {
             {
                 Phase ph(ctx, PH_KMVM);
@@ -956,13 +970,20 @@ int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol
             ++it;
             ++since;
             const bool last = it >= ctx->opts.max_iter;
+            bool applied = false;
             if (it % ctx->opts.check_every == 0 || last) {
                 KRR_TRY_CUDA(cudaMemcpyAsync(ctx->cg_host, ctx->cg, sizeof(CGScalars),
                                              cudaMemcpyDeviceToHost, ctx->stream));
                 if (form == 1)
                     KRR_TRY_CUDA(cudaMemcpyAsync(tc_err_host, tc_err_dev, sizeof(int),
                                                  cudaMemcpyDeviceToHost, ctx->stream));
-                KRR_TRY_CUDA(cudaStreamSynchronize(ctx->stream));
+                // The apply of this residual is queued before the host waits for the scalars: the GPU
+                // works while the host decides, and in all but the few iterations that replace the
+                // residual the apply is the one that is needed.
+                KRR_TRY_CUDA(cudaEventRecord(ctx->cg_read, ctx->stream));
+                KRR_RET(apply());
+                applied = true;
+                KRR_TRY_CUDA(cudaEventSynchronize(ctx->cg_read));
                 if (form == 1 && *tc_err_host) {
                     status = KRR_E_TIMEOUT;
                     fail(ctx, status, "tensor-core product: a bounded wait timed out");
@@ -1050,24 +1071,16 @@ int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol
                         continue;
                     }
                     KRR_RET(launch_cg_set_active(ctx, act.data(), nrhs));
+                    applied = false;   // the residual has been replaced
                 }
             }
-            {
-                Phase ph(ctx, PH_APPLY);
-                if (ctx->opts.no_precond)
-                    KRR_RET(hp ? launch_identity_apply64(ctx, rr64, nrhs, z64, part3)
-                               : launch_identity_apply(ctx, r, nrhs, z, part3));
-                else if (hp)
-                    KRR_RET(launch_apply_precond64(ctx, rr64, nrhs, z64, part3));
-                else
-                    KRR_RET(launch_apply_precond(ctx, r, nrhs, z, part3));
-            }
+            if (!applied) KRR_RET(apply());
             {
                 Phase ph(ctx, PH_CGVEC);
                 if (hp)
                     KRR_RET(launch_cg64_beta_p(ctx, p64, z64, nrhs, part3));
                 else
-                    KRR_RET(launch_cg_beta_p(ctx, p, z, nrhs, part3));
+                    KRR_RET(launch_cg_beta_p(ctx, p, z, nrhs, part3, !ctx->opts.no_precond));
             }
         }
         inf.iters = it;

@@ -38,6 +38,30 @@ __device__ __forceinline__ void block_sum_store(double v, double* part, int q) {
     }
 }
 
+// True in every thread of the grid's last block to get here: the blocks' global writes before the
+// call are then visible to it.  *ticket starts at 0 and is 0 again afterwards.
+__device__ __forceinline__ bool last_block(unsigned* ticket) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (last) *ticket = 0;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// sum of column q's per-block partials, in every lane (read past L1: another block of the same launch
+// may have written them)
+__device__ __forceinline__ double warp_sum_parts(const double* __restrict__ part, int nblk, int q) {
+    const int lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (int b = lane; b < nblk; b += 32) s += __ldcg(part + (size_t)q * nblk + b);
+    return warp_sum(s);
+}
+
 __global__ void __launch_bounds__(VT)
 k_dot_part(const float* __restrict__ A, const float* __restrict__ B, long long n, int nrhs,
            double* __restrict__ part) {
@@ -137,7 +161,7 @@ k_gemv_t(const float* __restrict__ F, long long n, int ldF, const float* __restr
             __syncthreads();
             if (c4 < ld4) {
                 const float4* fp = F4 + b0 * ld4 + c4;
-                constexpr int U = 8;   // rows whose loads are in flight together
+                constexpr int U = NQ > 4 ? 4 : 8;   // rows whose loads are in flight together
                 int i = 0;
                 for (; i + U <= nb; i += U) {
                     float4 f[U];
@@ -234,7 +258,7 @@ template <int NQ>
 __global__ void __launch_bounds__(VT)
 k_gemv_n_apply(const float* __restrict__ F, long long n, int k, int ldF, const double* __restrict__ v,
                const float* __restrict__ R, long long ldr, float inv_beta, float* __restrict__ Z,
-               double* __restrict__ rz_part) {
+               double* __restrict__ rz_part, CGScalars* cg, int q0) {
     extern __shared__ float4 sv4[];   // NQ x ld4
     const int ld4 = ldF >> 2;
     for (int e = threadIdx.x; e < NQ * ld4; e += VT) {
@@ -304,31 +328,50 @@ k_gemv_n_apply(const float* __restrict__ F, long long n, int k, int ldF, const d
     if (rz_part) {
 #pragma unroll
         for (int q = 0; q < NQ; ++q) block_sum_store(lane == 0 ? rz[q] : 0.0, rz_part, q);
+        // the last block forms the columns' b = rz_new / rz (b = 0 for finished columns: p restarts
+        // from z); rz itself is replaced when p is updated, so that this pass may be repeated
+        if (cg && last_block(&cg->ticket[0])) {
+            for (int q = w; q < NQ; q += VT / 32) {
+                const double s = warp_sum_parts(rz_part, gridDim.x, q);
+                if (lane == 0) {
+                    const double z = cg->rz[q0 + q];
+                    cg->b[q0 + q] = (cg->active[q0 + q] && z != 0.0 && isfinite(s)) ? s / z : 0.0;
+                    cg->rz_new[q0 + q] = s;
+                }
+            }
+        }
     }
 }
 
 typedef void (*gemv_t_fn)(const float*, long long, int, const float*, long long, long long, double*);
 typedef void (*gemv_n_fn)(const float*, long long, int, int, const double*, const float*, long long,
-                          float, float*, double*);
+                          float, float*, double*, CGScalars*, int);
+constexpr int AP_NQ = 8;   // most right-hand sides per pass over F
 
 // Z = M^{-1} R for nrhs columns.  When rz_part is non-null it receives per-block partial
-// sums of R.Z laid out [q][blk] with vec_blocks(n) blocks per column.
-int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, double* rz_part) {
+// sums of R.Z laid out [q][blk] with vec_blocks(n) blocks per column; with_beta also forms the
+// recurrence's b and rz_new from them.
+int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, double* rz_part, bool with_beta) {
     const long long n = ctx->n;
     const int k = ctx->k_eff, ldF = ctx->ldF;
     const int nb = vec_blocks(ctx, n);
     const long long rows_per = ceil_div(n, nb);
     double *upart, *u, *u1, *v;
-    KRR_RET(bufT(ctx, "ap_upart", (size_t)nb * 4 * ldF, &upart));
-    KRR_RET(bufT(ctx, "ap_u", (size_t)4 * k, &u));
-    KRR_RET(bufT(ctx, "ap_u1", (size_t)4 * k, &u1));
-    KRR_RET(bufT(ctx, "ap_v", (size_t)4 * k, &v));
+    const int mq = std::min(AP_NQ, nrhs);
+    KRR_RET(bufT(ctx, "ap_upart", (size_t)nb * mq * ldF, &upart));
+    KRR_RET(bufT(ctx, "ap_u", (size_t)mq * k, &u));
+    KRR_RET(bufT(ctx, "ap_u1", (size_t)mq * k, &u1));
+    KRR_RET(bufT(ctx, "ap_v", (size_t)mq * k, &v));
     const float inv_beta = (float)(1.0 / ctx->beta);
-    for (int q0 = 0; q0 < nrhs; q0 += 4) {
-        const int nq = std::min(4, nrhs - q0);
-        gemv_t_fn gt = nq == 1 ? &k_gemv_t<1> : nq == 2 ? &k_gemv_t<2> : nq == 3 ? &k_gemv_t<3> : &k_gemv_t<4>;
-        gemv_n_fn gn = nq == 1 ? &k_gemv_n_apply<1> : nq == 2 ? &k_gemv_n_apply<2>
-                     : nq == 3 ? &k_gemv_n_apply<3> : &k_gemv_n_apply<4>;
+    static const gemv_t_fn gts[AP_NQ] = {&k_gemv_t<1>, &k_gemv_t<2>, &k_gemv_t<3>, &k_gemv_t<4>,
+                                         &k_gemv_t<5>, &k_gemv_t<6>, &k_gemv_t<7>, &k_gemv_t<8>};
+    static const gemv_n_fn gns[AP_NQ] = {&k_gemv_n_apply<1>, &k_gemv_n_apply<2>, &k_gemv_n_apply<3>,
+                                         &k_gemv_n_apply<4>, &k_gemv_n_apply<5>, &k_gemv_n_apply<6>,
+                                         &k_gemv_n_apply<7>, &k_gemv_n_apply<8>};
+    for (int q0 = 0; q0 < nrhs; q0 += AP_NQ) {
+        const int nq = std::min(AP_NQ, nrhs - q0);
+        const gemv_t_fn gt = gts[nq - 1];
+        const gemv_n_fn gn = gns[nq - 1];
         const float* Rq = R + (size_t)q0 * n;
         float* Zq = Z + (size_t)q0 * n;
         gt<<<nb, VT, 0, ctx->stream>>>(ctx->F, n, ldF, Rq, n, rows_per, upart);
@@ -344,7 +387,8 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
             KRR_RET(allow_max_dynamic_smem(ctx, (const void*)gn));
         }
         gn<<<nb, VT, smem, ctx->stream>>>(ctx->F, n, k, ldF, v, Rq, n, inv_beta, Zq,
-                                          rz_part ? rz_part + (size_t)q0 * nb : nullptr);
+                                          rz_part ? rz_part + (size_t)q0 * nb : nullptr,
+                                          rz_part && with_beta ? ctx->cg : nullptr, q0);
         KRR_CHECK_LAUNCH();
     }
     return KRR_OK;
@@ -353,19 +397,8 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
 // ------------------------------------------------------------------ PCG recurrences
 // The scalar kernels run one warp per right-hand side: the warp sums that column's
 // per-block partials (FP64) and lane 0 applies the recurrence.
-__device__ __forceinline__ double warp_sum_parts(const double* __restrict__ part, int nblk, int q) {
-    const int lane = threadIdx.x & 31;
-    double s = 0.0;
-    for (int b = lane; b < nblk; b += 32) s += part[(size_t)q * nblk + b];
-    return warp_sum(s);
-}
-
-// a_q = rz_q / (p_q . q_q) for active columns; zero otherwise.
-__global__ void k_cg_alpha(CGScalars* cg, const double* __restrict__ part, int nblk, int nrhs) {
-    const int q = threadIdx.x >> 5;
-    if (q >= nrhs) return;
-    const double s = warp_sum_parts(part, nblk, q);
-    if ((threadIdx.x & 31) != 0) return;
+// a_q = rz_q / (p_q . q_q) for active columns; zero otherwise (one warp; s = p_q . q_q).
+__device__ __forceinline__ void cg_alpha(CGScalars* cg, int q, double s) {
     cg->pq[q] = s;
     double a = 0.0;
     if (cg->active[q]) {
@@ -378,12 +411,58 @@ __global__ void k_cg_alpha(CGScalars* cg, const double* __restrict__ part, int n
     }
     cg->a[q] = a;
 }
+__global__ void k_cg_alpha(CGScalars* cg, const double* __restrict__ part, int nblk, int nrhs) {
+    const int q = threadIdx.x >> 5;
+    if (q >= nrhs) return;
+    const double s = warp_sum_parts(part, nblk, q);
+    if ((threadIdx.x & 31) == 0) cg_alpha(cg, q, s);
+}
+// p . q and, in the last block, the step lengths: one launch instead of two in every iteration
+__global__ void __launch_bounds__(VT)
+k_cg_dot_alpha(const float* __restrict__ p, const float* __restrict__ qv, long long n, int nrhs, CGScalars* cg,
+               double* __restrict__ part) {
+    for (int q = 0; q < nrhs; ++q) {
+        double s = 0.0;
+        for (long long i = (long long)blockIdx.x * VT + threadIdx.x; i < n; i += (long long)gridDim.x * VT)
+            s += (double)p[q * n + i] * (double)qv[q * n + i];
+        block_sum_store(s, part, q);
+    }
+    if (!last_block(&cg->ticket[1])) return;
+    for (int q = threadIdx.x >> 5; q < nrhs; q += VT / 32) {
+        const double s = warp_sum_parts(part, gridDim.x, q);
+        if ((threadIdx.x & 31) == 0) cg_alpha(cg, q, s);
+    }
+}
 
-// x += a p; r -= a q; partial r.r
+// rr_q = s (recursive residual); a non-finite one ends the column, and with tol2 > 0 so does
+// rr_q <= tol2 rr0_q.  Returns whether the column goes on.
+__device__ __forceinline__ bool cg_check(CGScalars* cg, int q, double s, double tol2) {
+    cg->rr[q] = s;
+    if (!isfinite(s)) {
+        cg->bad = 1;
+        cg->active[q] = 0;
+    }
+    if (tol2 > 0.0 && cg->active[q] && !(s > tol2 * cg->rr0[q])) cg->active[q] = 0;
+    return cg->active[q] != 0;
+}
+__global__ void k_cg_check(CGScalars* cg, const double* __restrict__ part, int nblk, int nrhs,
+                           double tol2) {
+    __shared__ int any;
+    if (threadIdx.x == 0) any = 0;
+    __syncthreads();
+    const int q = threadIdx.x >> 5;
+    if (q < nrhs) {
+        const double s = warp_sum_parts(part, nblk, q);
+        if ((threadIdx.x & 31) == 0 && cg_check(cg, q, s, tol2)) atomicOr(&any, 1);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) cg->all_done = any ? 0 : 1;
+}
+// x += a p; r -= a q; r.r and, in the last block, the check above
 __global__ void __launch_bounds__(VT)
 k_cg_update_xr(float* __restrict__ x, float* __restrict__ r, const float* __restrict__ p,
-               const float* __restrict__ qv, long long n, int nrhs, const CGScalars* __restrict__ cg,
-               double* __restrict__ part) {
+               const float* __restrict__ qv, long long n, int nrhs, CGScalars* cg,
+               double* __restrict__ part, double tol2) {
     for (int q = 0; q < nrhs; ++q) {
         const float a = (float)cg->a[q];
         double s = 0.0;
@@ -396,26 +475,13 @@ k_cg_update_xr(float* __restrict__ x, float* __restrict__ r, const float* __rest
         }
         block_sum_store(s, part, q);
     }
-}
-
-// rr_q = sum part (recursive residual); columns with tol2 > 0 stop once rr_q <= tol2 rr0_q.
-__global__ void k_cg_check(CGScalars* cg, const double* __restrict__ part, int nblk, int nrhs,
-                           double tol2) {
+    if (!last_block(&cg->ticket[2])) return;
     __shared__ int any;
     if (threadIdx.x == 0) any = 0;
     __syncthreads();
-    const int q = threadIdx.x >> 5;
-    if (q < nrhs) {
-        const double s = warp_sum_parts(part, nblk, q);
-        if ((threadIdx.x & 31) == 0) {
-            cg->rr[q] = s;
-            if (!isfinite(s)) {
-                cg->bad = 1;
-                cg->active[q] = 0;
-            }
-            if (tol2 > 0.0 && cg->active[q] && !(s > tol2 * cg->rr0[q])) cg->active[q] = 0;
-            if (cg->active[q]) atomicOr(&any, 1);
-        }
+    for (int q = threadIdx.x >> 5; q < nrhs; q += VT / 32) {
+        const double s = warp_sum_parts(part, gridDim.x, q);
+        if ((threadIdx.x & 31) == 0 && cg_check(cg, q, s, tol2)) atomicOr(&any, 1);
     }
     __syncthreads();
     if (threadIdx.x == 0) cg->all_done = any ? 0 : 1;
@@ -432,10 +498,11 @@ __global__ void k_cg_beta(CGScalars* cg, const double* __restrict__ part, int nb
     cg->rz[q] = s;
 }
 
-// p = z + b p
+// p = z + b p; with_beta (b came with the apply): rz = rz_new, which nothing here reads
 __global__ void __launch_bounds__(VT)
-k_cg_update_p(float* __restrict__ p, const float* __restrict__ z, long long n, int nrhs,
-              const CGScalars* __restrict__ cg) {
+k_cg_update_p(float* __restrict__ p, const float* __restrict__ z, long long n, int nrhs, CGScalars* cg,
+              bool with_beta) {
+    if (with_beta && blockIdx.x == 0 && (int)threadIdx.x < nrhs) cg->rz[threadIdx.x] = cg->rz_new[threadIdx.x];
     const long long tot = n * nrhs;
     for (long long e = (long long)blockIdx.x * VT + threadIdx.x; e < tot; e += (long long)gridDim.x * VT) {
         const int q = (int)(e / n);
@@ -503,9 +570,7 @@ int launch_cg_start(krr_ctx* ctx, const float* r, const float* z, int nrhs, doub
 
 int launch_cg_alpha(krr_ctx* ctx, const float* p, const float* q, int nrhs, double* part) {
     const int nb = vec_blocks(ctx, ctx->n);
-    k_dot_part<<<nb, VT, 0, ctx->stream>>>(p, q, ctx->n, nrhs, part);
-    KRR_CHECK_LAUNCH();
-    k_cg_alpha<<<1, 32 * nrhs, 0, ctx->stream>>>(ctx->cg, part, nb, nrhs);
+    k_cg_dot_alpha<<<nb, VT, 0, ctx->stream>>>(p, q, ctx->n, nrhs, ctx->cg, part);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -513,18 +578,18 @@ int launch_cg_alpha(krr_ctx* ctx, const float* p, const float* q, int nrhs, doub
 int launch_cg_update_xr(krr_ctx* ctx, float* x, float* r, const float* p, const float* q, int nrhs,
                         double* part, double tol2) {
     const int nb = vec_blocks(ctx, ctx->n);
-    k_cg_update_xr<<<nb, VT, 0, ctx->stream>>>(x, r, p, q, ctx->n, nrhs, ctx->cg, part);
-    KRR_CHECK_LAUNCH();
-    k_cg_check<<<1, 32 * nrhs, 0, ctx->stream>>>(ctx->cg, part, nb, nrhs, tol2);
+    k_cg_update_xr<<<nb, VT, 0, ctx->stream>>>(x, r, p, q, ctx->n, nrhs, ctx->cg, part, tol2);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
 
-int launch_cg_beta_p(krr_ctx* ctx, float* p, const float* z, int nrhs, const double* rz_part) {
+int launch_cg_beta_p(krr_ctx* ctx, float* p, const float* z, int nrhs, const double* rz_part, bool with_beta) {
     const int nb = vec_blocks(ctx, ctx->n);
-    k_cg_beta<<<1, 32 * nrhs, 0, ctx->stream>>>(ctx->cg, rz_part, nb, nrhs);
-    KRR_CHECK_LAUNCH();
-    k_cg_update_p<<<nb, VT, 0, ctx->stream>>>(p, z, ctx->n, nrhs, ctx->cg);
+    if (!with_beta) {
+        k_cg_beta<<<1, 32 * nrhs, 0, ctx->stream>>>(ctx->cg, rz_part, nb, nrhs);
+        KRR_CHECK_LAUNCH();
+    }
+    k_cg_update_p<<<nb, VT, 0, ctx->stream>>>(p, z, ctx->n, nrhs, ctx->cg, with_beta);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }

@@ -65,6 +65,7 @@ struct CGScalars {
     int all_done;
     int bad;            // a non-finite or non-positive curvature was met
     int tc_err;         // host mirror only: the tensor-core product's error word
+    unsigned ticket[3]; // blocks that have finished, of the passes whose last block forms scalars
 };
 
 struct Buf {
@@ -121,6 +122,7 @@ struct krr_ctx {
     unsigned char* FB = nullptr;   // tensor-core features of X (column role)
     krr::CGScalars* cg = nullptr;
     krr::CGScalars* cg_host = nullptr;   // pinned mirror
+    cudaEvent_t cg_read = nullptr;       // the mirror has been written
 
     // ---- phase timers (off unless krr_profile_enable)
     bool prof = false;
@@ -370,7 +372,8 @@ int launch_set_identity(krr_ctx* ctx, double* A, int k);
 int launch_add_diag(krr_ctx* ctx, double* A, int k, double v);
 
 // cg.cu
-int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, double* rz_part_out);
+int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, double* rz_part_out,
+                         bool with_beta = false);
 // b = (float) a; b = (double) a; y += x (tot elements)
 int launch_convert(krr_ctx* ctx, const double* a, float* b, long long tot);
 int launch_convert_up(krr_ctx* ctx, const float* a, double* b, long long tot);
