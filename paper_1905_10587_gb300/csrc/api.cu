@@ -226,21 +226,23 @@ static int build_from_anchors(krr_ctx* ctx, const int* S_dev, int k_eff) {
     KRR_RET(bufT(ctx, "L1", (size_t)k_eff * k_eff, &L1));
     KRR_RET(bufT(ctx, "L1inv", (size_t)k_eff * k_eff, &L1inv));
     int info = 0;
+    double* dinv;
+    KRR_RET(potrf_dinv(ctx, k_eff, &dinv));
     {
         Phase ph_chol(ctx, PH_CHOL);
         KRR_RET(launch_kss(ctx, ctx->XS, k_eff, d, ctx->sigma, L1));
-        KRR_RET(launch_potrf(ctx, L1, k_eff, &info, ctx->opts.pivot_tol));
+        KRR_RET(launch_potrf(ctx, L1, k_eff, &info, dinv, ctx->opts.pivot_tol));
         if (info != 0) {
             const int keep = info - 1;
             if (keep < 1) return fail(ctx, KRR_E_NONFINITE, "first anchor pivot is not positive");
             k_eff = keep;
             ctx->k_eff = keep;
             KRR_RET(launch_kss(ctx, ctx->XS, k_eff, d, ctx->sigma, L1));   // prefix of the same S
-            KRR_RET(launch_potrf(ctx, L1, k_eff, &info, 0.0));
+            KRR_RET(launch_potrf(ctx, L1, k_eff, &info, dinv, 0.0));
             if (info != 0) return fail(ctx, KRR_E_NOTSPD, "Cholesky of K_SS failed");
         }
         KRR_RET(launch_set_identity(ctx, L1inv, k_eff));
-        KRR_RET(launch_trsm_lower(ctx, L1, L1inv, k_eff));
+        KRR_RET(launch_tri_inverse(ctx, L1, dinv, L1inv, k_eff));
     }
 
     // F = K(X, X_S) L1^{-T}  (n x ldF)
@@ -264,12 +266,12 @@ static int build_from_anchors(krr_ctx* ctx, const int* S_dev, int k_eff) {
         KRR_RET(launch_gram(ctx, ctx->F, n, k_eff, ctx->ldF, ctx->beta, G));
     }
     Phase ph_chol2(ctx, PH_CHOL);   // until the end of the build
-    KRR_RET(launch_potrf(ctx, G, k_eff, &info));
+    KRR_RET(launch_potrf(ctx, G, k_eff, &info, dinv));
     if (info != 0) return fail(ctx, KRR_E_NOTSPD, "Cholesky of beta I + F^T F failed");
     KRR_RET(bufT(ctx, "T2", (size_t)k_eff * k_eff, &ctx->T2));
     KRR_RET(bufT(ctx, "T2t", (size_t)k_eff * k_eff, &ctx->T2t));
     KRR_RET(launch_set_identity(ctx, ctx->T2, k_eff));
-    KRR_RET(launch_trsm_lower(ctx, G, ctx->T2, k_eff));
+    KRR_RET(launch_tri_inverse(ctx, G, dinv, ctx->T2, k_eff));
     KRR_RET(launch_transpose64(ctx, ctx->T2, ctx->T2t, k_eff));
     return KRR_OK;
 }

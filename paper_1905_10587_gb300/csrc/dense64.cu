@@ -1,6 +1,6 @@
 // FP64 k x k linear algebra of the preconditioner build (Algorithm 3, Eq. (10)):
-// the anchor kernel block K_SS, blocked right-looking Cholesky, triangular
-// inversion by blocked forward substitution, and small helpers.  All matrices are
+// the anchor kernel block K_SS, blocked right-looking Cholesky with inverted diagonal
+// blocks, triangular inversion by blocks, and small helpers.  All matrices are
 // row-major k x k.  k is at most a few thousand, so these run a few hundred
 // small launches; GB300's FP64 rate, not memory, bounds them.
 #include "internal.cuh"
@@ -33,85 +33,125 @@ int launch_kss(krr_ctx* ctx, const float* XS, int k, int d, double sigma, double
     return KRR_OK;
 }
 
-// ---- unblocked Cholesky of the nb x nb diagonal block at (j0, j0); one CTA of NB x NB threads.
-__global__ void __launch_bounds__(NB * NB)
-k_potf2(double* __restrict__ A, int k, int j0, int nb, double tau, int* __restrict__ info) {
-    __shared__ double s[NB][NB + 1];
-    const int r = threadIdx.y, c = threadIdx.x;
-    s[r][c] = (r < nb && c < nb) ? A[(size_t)(j0 + r) * k + j0 + c] : 0.0;
+// FP64 on this GPU issues one warp instruction per ~70 cycles and SM quarter, so what counts in
+// these small kernels is the number of dependent FP64 instructions of a thread and how many SMs
+// share the work, not memory.  Hence: the diagonal block is factored and inverted in one kernel
+// with one reciprocal per column (no divisions or square roots in the elimination; 1024 threads
+// that each took the column's square root needed 130 us a block), the blocks below and right of it
+// are multiplied by that inverse, one output per thread (a substitution per thread needed 37 to
+// 45 us), and trailing updates use 16 x 16 tiles with one output per thread.  Both factorizations
+// and inverses of a build with k = 200 went from 3.31 to 0.89 ms, with k = 100 from 1.66 to 0.46 ms.
+
+// 1 / d to FP64 rounding (a few ulp) from the FP32 reciprocal and two Newton steps; d is a pivot
+// in the normal FP32 range (0 and non-finite pivots are refused before).
+__device__ __forceinline__ double recip64(double d) {
+    int ex;
+    const double m = frexp(d, &ex);                // [0.5, 1): the FP32 seed neither over- nor underflows
+    double x = (double)(1.0f / (float)m);
+    x = fma(x, fma(-m, x, 1.0), x);
+    x = fma(x, fma(-m, x, 1.0), x);
+    return ldexp(x, -ex);
+}
+
+// Cholesky of the nb x nb diagonal block at (j0, j0), and its inverse into Linv (NB x NB, row
+// major, lower; identity-padded): A_jj = L L^T.  Elimination keeps A_jj = U^T D U unscaled
+// (v_r = pivot column, d its pivot): a_rc -= v_r (v_c / d), and the same row operations on the
+// identity give the unit inverse; L and its inverse follow from both by the d^(1/2) in parallel.
+// Threads (x, y) of 32 x 8 own column x of rows y, y + 8, ...
+constexpr int PF_Y = 8;
+__global__ void __launch_bounds__(NB * PF_Y)
+k_potf2(double* __restrict__ A, int k, int j0, int nb, double tau, int* __restrict__ info,
+        double* __restrict__ Linv) {
+    __shared__ double s[NB][NB + 1], ei[NB][NB + 1], w[NB], sd[NB];
+    const int c = threadIdx.x, y = threadIdx.y;
+#pragma unroll
+    for (int r = y; r < NB; r += PF_Y) {
+        s[r][c] = (r < nb && c < nb) ? A[(size_t)(j0 + r) * k + j0 + c] : (r == c ? 1.0 : 0.0);
+        ei[r][c] = r == c ? 1.0 : 0.0;
+    }
     __syncthreads();
     for (int m = 0; m < nb; ++m) {
         const double piv = s[m][m];
         const bool bad = !(piv > tau) || !isfinite(piv);
         if (bad) {
-            if (r == 0 && c == 0) atomicCAS(info, 0, j0 + m + 1);
+            if (y == 0 && c == 0) atomicCAS(info, 0, j0 + m + 1);
             return;   // uniform: every thread sees the same s[m][m]
         }
-        const double dm = sqrt(piv);
-        __syncthreads();
-        if (c == m && r >= m) s[r][m] = (r == m) ? dm : s[r][m] / dm;
-        __syncthreads();
-        if (r > m && c > m && c <= r) s[r][c] -= s[r][m] * s[c][m];
-        __syncthreads();
-    }
-    if (r < nb && c < nb) A[(size_t)(j0 + r) * k + j0 + c] = (c <= r) ? s[r][c] : 0.0;
-}
-
-// ---- panel solve: rows i >= j0+nb, A[i, j0:j0+nb] <- A[i, j0:j0+nb] L_jj^{-T}
-__global__ void __launch_bounds__(128)
-k_potrf_panel(double* __restrict__ A, int k, int j0, int nb) {
-    __shared__ double L[NB][NB + 1];
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-        const int r = e / NB, c = e - r * NB;
-        L[r][c] = (r < nb && c < nb) ? A[(size_t)(j0 + r) * k + j0 + c] : 0.0;
-    }
-    __syncthreads();
-    const int i = j0 + nb + blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= k) return;
-    double x[NB];
-#pragma unroll
-    for (int c = 0; c < NB; ++c) x[c] = (c < nb) ? A[(size_t)i * k + j0 + c] : 0.0;
-#pragma unroll
-    for (int c = 0; c < NB; ++c) {
-        if (c < nb) {
-            double v = x[c];
-#pragma unroll
-            for (int m = 0; m < c; ++m) v -= x[m] * L[c][m];
-            x[c] = v / L[c][c];
+        if (y == 0) {                              // one warp: w_c = v_c / d
+            const double inv = recip64(piv);
+            w[c] = c > m ? s[c][m] * inv : 0.0;
         }
-    }
+        __syncthreads();
 #pragma unroll
-    for (int c = 0; c < NB; ++c)
-        if (c < nb) A[(size_t)i * k + j0 + c] = x[c];
+        for (int r = y; r < NB; r += PF_Y) {
+            if (r > m) {
+                if (c > m && c <= r) s[r][c] = fma(-s[r][m], w[c], s[r][c]);
+                else if (c <= m) ei[r][c] = fma(-w[r], ei[m][c], ei[r][c]);
+            }
+        }
+        __syncthreads();
+    }
+    if (y == 0) sd[c] = sqrt(s[c][c]);             // pivots (1 in the padding)
+    __syncthreads();
+    if (y == 0) w[c] = 1.0 / sd[c];
+    __syncthreads();
+#pragma unroll
+    for (int r = y; r < NB; r += PF_Y) {
+        if (r < nb && c < nb)
+            A[(size_t)(j0 + r) * k + j0 + c] = c < r ? s[r][c] * w[c] : c == r ? sd[c] : 0.0;
+        Linv[r * NB + c] = c <= r ? ei[r][c] * w[r] : 0.0;
+    }
 }
 
-// ---- trailing update: A[i, j] -= sum_m A[i, j0+m] A[j, j0+m]  for blocks (bi >= bj) past j0+nb
-__global__ void __launch_bounds__(256)
+// ---- rows i >= j0 + nb: A[i, j0 : j0 + nb] <- A[i, j0 : j0 + nb] L_jj^{-T}, one output a thread
+// (a warp per row: its inputs are read by the warp before any of its outputs is written)
+__global__ void __launch_bounds__(128)
+k_potrf_panel(double* __restrict__ A, int k, int j0, int nb, const double* __restrict__ Linv) {
+    __shared__ double L[NB][NB + 1];
+    __shared__ double x[4][NB];
+    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) L[e / NB][e % NB] = Linv[e];
+    const int c = threadIdx.x & 31, wr = threadIdx.x >> 5;
+    const int i = j0 + nb + blockIdx.x * 4 + wr;
+    x[wr][c] = (i < k && c < nb) ? A[(size_t)i * k + j0 + c] : 0.0;
+    __syncthreads();
+    if (i >= k || c >= nb) return;
+    double v0 = 0.0, v1 = 0.0;
+    for (int m = 0; m <= c; m += 2) {              // Linv[c][m] is 0 beyond m = c
+        v0 = fma(x[wr][m], L[c][m], v0);
+        if (m + 1 < NB) v1 = fma(x[wr][m + 1], L[c][m + 1], v1);
+    }
+    A[(size_t)i * k + j0 + c] = v0 + v1;
+}
+
+// ---- trailing update: A[i, j] -= sum_m A[i, j0+m] A[j, j0+m]  for 16 x 16 tiles (bi >= bj) past j0+nb
+constexpr int DT = 16;
+__global__ void __launch_bounds__(DT * DT)
 k_potrf_update(double* __restrict__ A, int k, int j0, int nb, int t0) {
-    // blockIdx.x enumerates lower-triangular block pairs of the trailing matrix
-    int p = blockIdx.x, bi = 0;
+    // blockIdx.x enumerates the lower-triangular tile pairs of the trailing matrix
+    const int p = blockIdx.x;
+    int bi = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
     while ((bi + 1) * (bi + 2) / 2 <= p) ++bi;
+    while (bi * (bi + 1) / 2 > p) --bi;
     const int bj = p - bi * (bi + 1) / 2;
-    const int r0 = t0 + bi * NB, c0 = t0 + bj * NB;
-    __shared__ double sa[NB][NB + 1];
-    __shared__ double sb[NB][NB + 1];
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
+    const int r0 = t0 + bi * DT, c0 = t0 + bj * DT;
+    __shared__ double sa[DT][NB + 1];
+    __shared__ double sb[DT][NB + 1];
+    for (int e = threadIdx.x; e < DT * NB; e += DT * DT) {
         const int r = e / NB, m = e - r * NB;
         sa[r][m] = (r0 + r < k && m < nb) ? A[(size_t)(r0 + r) * k + j0 + m] : 0.0;
         sb[r][m] = (c0 + r < k && m < nb) ? A[(size_t)(c0 + r) * k + j0 + m] : 0.0;
     }
     __syncthreads();
-    const int c = threadIdx.x & 31, rq = threadIdx.x >> 5;   // 8 row groups of 4
+    const int c = threadIdx.x % DT, r = threadIdx.x / DT;
+    const int gi = r0 + r, gj = c0 + c;
+    if (gi >= k || gj >= k || gj > gi) return;
+    double v0 = 0.0, v1 = 0.0;
 #pragma unroll
-    for (int rr = 0; rr < 4; ++rr) {
-        const int r = rq * 4 + rr;
-        const int gi = r0 + r, gj = c0 + c;
-        if (gi >= k || gj >= k || gj > gi) continue;
-        double s = 0.0;
-#pragma unroll 8
-        for (int m = 0; m < NB; ++m) s = fma(sa[r][m], sb[c][m], s);
-        A[(size_t)gi * k + gj] -= s;
+    for (int m = 0; m < NB; m += 2) {
+        v0 = fma(sa[r][m], sb[c][m], v0);
+        v1 = fma(sa[r][m + 1], sb[c][m + 1], v1);
     }
+    A[(size_t)gi * k + gj] -= v0 + v1;
 }
 
 __global__ void k_zero_upper(double* A, int k) {
@@ -121,20 +161,24 @@ __global__ void k_zero_upper(double* A, int k) {
     if (c > r) A[e] = 0.0;
 }
 
-int launch_potrf(krr_ctx* ctx, double* A, int k, int* info_host, double tau) {
+static int nblocks(int k) { return (k + NB - 1) / NB; }
+
+// dinv receives the inverses of the diagonal blocks of L (nblocks(k) x NB x NB).
+int launch_potrf(krr_ctx* ctx, double* A, int k, int* info_host, double* dinv, double tau) {
     int* info;
     KRR_RET(bufT(ctx, "potrf_info", 1, &info));
     KRR_TRY_CUDA(cudaMemsetAsync(info, 0, sizeof(int), ctx->stream));
     for (int j0 = 0; j0 < k; j0 += NB) {
         const int nb = std::min(NB, k - j0);
-        k_potf2<<<1, dim3(NB, NB), 0, ctx->stream>>>(A, k, j0, nb, tau, info);
+        double* Lj = dinv + (size_t)(j0 / NB) * NB * NB;
+        k_potf2<<<1, dim3(NB, PF_Y), 0, ctx->stream>>>(A, k, j0, nb, tau, info, Lj);
         KRR_CHECK_LAUNCH();
         const int rest = k - j0 - nb;
         if (rest <= 0) break;
-        k_potrf_panel<<<ceil_div(rest, 128), 128, 0, ctx->stream>>>(A, k, j0, nb);
+        k_potrf_panel<<<ceil_div(rest, 4), 128, 0, ctx->stream>>>(A, k, j0, nb, Lj);
         KRR_CHECK_LAUNCH();
-        const int tb = (rest + NB - 1) / NB;
-        k_potrf_update<<<tb * (tb + 1) / 2, 256, 0, ctx->stream>>>(A, k, j0, nb, j0 + nb);
+        const int tb = (rest + DT - 1) / DT;
+        k_potrf_update<<<tb * (tb + 1) / 2, DT * DT, 0, ctx->stream>>>(A, k, j0, nb, j0 + nb);
         KRR_CHECK_LAUNCH();
     }
     k_zero_upper<<<ceil_div((long long)k * k, 256), 256, 0, ctx->stream>>>(A, k);
@@ -144,76 +188,97 @@ int launch_potrf(krr_ctx* ctx, double* A, int k, int* info_host, double tau) {
     return KRR_OK;
 }
 
-// ---- solve L X = B in place, right-looking by 32-row blocks.  B = I gives X = L^{-1}
-// (lower triangular), so only columns < j0 + nb carry nonzeros at step j0.
-__global__ void __launch_bounds__(128)
-k_trsm_diag(const double* __restrict__ L, double* __restrict__ B, int k, int j0, int nb,
-            int ncols) {
-    __shared__ double sl[NB][NB + 1];
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-        const int r = e / NB, c = e - r * NB;
-        sl[r][c] = (r < nb && c < nb) ? L[(size_t)(j0 + r) * k + j0 + c] : 0.0;
-    }
-    __syncthreads();
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= ncols) return;
-    double x[NB];
-#pragma unroll
-    for (int r = 0; r < NB; ++r) x[r] = (r < nb) ? B[(size_t)(j0 + r) * k + col] : 0.0;
-#pragma unroll
-    for (int r = 0; r < NB; ++r) {
-        if (r < nb) {
-            double v = x[r];
-#pragma unroll
-            for (int m = 0; m < r; ++m) v -= sl[r][m] * x[m];
-            x[r] = v / sl[r][r];
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < NB; ++r)
-        if (r < nb) B[(size_t)(j0 + r) * k + col] = x[r];
+int potrf_dinv(krr_ctx* ctx, int k, double** dinv) {
+    return bufT(ctx, "potrf_dinv", (size_t)nblocks(k) * NB * NB, dinv);
 }
 
-// B[i, c] -= sum_m L[i, j0+m] B[j0+m, c]  for i >= j0+nb, c < ncols.  CTA: 32 rows x 64 cols.
-__global__ void __launch_bounds__(256)
-k_trsm_update(const double* __restrict__ L, double* __restrict__ B, int k, int j0, int nb,
-              int ncols) {
+// ---- X = L^{-1} (lower) by 32-row blocks: at step j0 the rows j0 .. of B hold the identity minus
+// what the blocks above contributed; X[j0:, c] = L_jj^{-1} B[j0:, c], then B[i, c] -= L[i, j0:] X[j0:, c]
+// for the rows below.  B starts as the identity, so only the columns c < j0 + nb are non-zero.
+// One output a thread; a block holds 32 rows x 8 columns, which it reads before it writes.
+constexpr int TD_C = 8;
+__global__ void __launch_bounds__(NB * TD_C)
+k_trinv_diag(const double* __restrict__ Linv, double* __restrict__ B, int k, int j0, int nb, int ncols) {
     __shared__ double sl[NB][NB + 1];
-    __shared__ double sx[NB][64 + 1];
-    const int r0 = j0 + nb + blockIdx.y * NB;
-    const int c0 = blockIdx.x * 64;
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
+    __shared__ double sx[NB][TD_C + 1];
+    for (int e = threadIdx.x; e < NB * NB; e += NB * TD_C) sl[e / NB][e % NB] = Linv[e];
+    const int c = threadIdx.x % TD_C, r = threadIdx.x / TD_C;
+    const int col = blockIdx.x * TD_C + c;
+    const bool ok = r < nb && col < ncols;
+    sx[r][c] = ok ? B[(size_t)(j0 + r) * k + col] : 0.0;
+    __syncthreads();
+    if (!ok) return;
+    double v0 = 0.0, v1 = 0.0;
+    for (int m = 0; m <= r; m += 2) {
+        v0 = fma(sl[r][m], sx[m][c], v0);
+        if (m + 1 < NB) v1 = fma(sl[r][m + 1], sx[m + 1][c], v1);
+    }
+    B[(size_t)(j0 + r) * k + col] = v0 + v1;
+}
+
+// B[i, c] -= sum_m L[i, j0+m] B[j0+m, c]  for i >= j0+nb, c < ncols, in 16 x 16 tiles
+__global__ void __launch_bounds__(DT * DT)
+k_trinv_update(const double* __restrict__ L, double* __restrict__ B, int k, int j0, int nb, int ncols) {
+    __shared__ double sl[DT][NB + 1];
+    __shared__ double sx[NB][DT + 1];
+    const int r0 = j0 + nb + blockIdx.y * DT, c0 = blockIdx.x * DT;
+    for (int e = threadIdx.x; e < DT * NB; e += DT * DT) {
         const int r = e / NB, m = e - r * NB;
         sl[r][m] = (r0 + r < k && m < nb) ? L[(size_t)(r0 + r) * k + j0 + m] : 0.0;
-    }
-    for (int e = threadIdx.x; e < NB * 64; e += blockDim.x) {
-        const int m = e / 64, c = e - m * 64;
-        sx[m][c] = (m < nb && c0 + c < ncols) ? B[(size_t)(j0 + m) * k + c0 + c] : 0.0;
+        const int m2 = e / DT, c = e - m2 * DT;
+        sx[m2][c] = (m2 < nb && c0 + c < ncols) ? B[(size_t)(j0 + m2) * k + c0 + c] : 0.0;
     }
     __syncthreads();
-    const int c = threadIdx.x & 63, rq = threadIdx.x >> 6;   // 4 groups of 8 rows
-    if (c0 + c >= ncols) return;
+    const int c = threadIdx.x % DT, r = threadIdx.x / DT;
+    if (r0 + r >= k || c0 + c >= ncols) return;
+    double v0 = 0.0, v1 = 0.0;
 #pragma unroll
-    for (int rr = 0; rr < 8; ++rr) {
-        const int r = rq * 8 + rr;
-        if (r0 + r >= k) break;
-        double s = 0.0;
-#pragma unroll 8
-        for (int m = 0; m < NB; ++m) s = fma(sl[r][m], sx[m][c], s);
-        B[(size_t)(r0 + r) * k + c0 + c] -= s;
+    for (int m = 0; m < NB; m += 2) {
+        v0 = fma(sl[r][m], sx[m][c], v0);
+        v1 = fma(sl[r][m + 1], sx[m + 1][c], v1);
     }
+    B[(size_t)(r0 + r) * k + c0 + c] -= v0 + v1;
 }
 
-int launch_trsm_lower(krr_ctx* ctx, const double* L, double* B, int k) {
+// Inverses of the diagonal blocks of a lower triangular L that launch_potrf did not make, one block
+// of threads each: forward elimination of [L_jj | I].
+__global__ void __launch_bounds__(NB * PF_Y)
+k_diag_inverse(const double* __restrict__ L, int k, double* __restrict__ dinv) {
+    __shared__ double s[NB][NB + 1], e[NB][NB + 1];
+    const int c = threadIdx.x, y = threadIdx.y, j0 = blockIdx.x * NB, nb = min(NB, k - j0);
+    for (int r = y; r < NB; r += PF_Y) {
+        s[r][c] = (r < nb && c < nb) ? L[(size_t)(j0 + r) * k + j0 + c] : (r == c ? 1.0 : 0.0);
+        e[r][c] = r == c ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    for (int m = 0; m < nb; ++m) {
+        if (y == 0 && c <= m) e[m][c] /= s[m][m];
+        __syncthreads();
+        for (int r = y; r < NB; r += PF_Y)
+            if (r > m && c <= m) e[r][c] = fma(-s[r][m], e[m][c], e[r][c]);
+        __syncthreads();
+    }
+    for (int r = y; r < NB; r += PF_Y) dinv[(size_t)blockIdx.x * NB * NB + r * NB + c] = c <= r ? e[r][c] : 0.0;
+}
+
+int launch_diag_inverse(krr_ctx* ctx, const double* L, int k, double* dinv) {
+    k_diag_inverse<<<nblocks(k), dim3(NB, PF_Y), 0, ctx->stream>>>(L, k, dinv);
+    KRR_CHECK_LAUNCH();
+    return KRR_OK;
+}
+
+// B (identity on entry) <- L^{-1}; dinv from launch_potrf on L or from launch_diag_inverse.
+int launch_tri_inverse(krr_ctx* ctx, const double* L, const double* dinv, double* B, int k) {
     for (int j0 = 0; j0 < k; j0 += NB) {
         const int nb = std::min(NB, k - j0);
-        const int ncols = j0 + nb;   // B = I: columns >= j0+nb are still zero in these rows
-        k_trsm_diag<<<ceil_div(ncols, 128), 128, 0, ctx->stream>>>(L, B, k, j0, nb, ncols);
+        const int ncols = j0 + nb;   // columns >= j0 + nb are still zero in these rows
+        k_trinv_diag<<<ceil_div(ncols, TD_C), NB * TD_C, 0, ctx->stream>>>(dinv + (size_t)(j0 / NB) * NB * NB, B, k,
+                                                                           j0, nb, ncols);
         KRR_CHECK_LAUNCH();
         const int rest = k - j0 - nb;
         if (rest <= 0) break;
-        dim3 grid(ceil_div(ncols, 64), ceil_div(rest, NB));
-        k_trsm_update<<<grid, 256, 0, ctx->stream>>>(L, B, k, j0, nb, ncols);
+        dim3 grid(ceil_div(ncols, DT), ceil_div(rest, DT));
+        k_trinv_update<<<grid, DT * DT, 0, ctx->stream>>>(L, B, k, j0, nb, ncols);
         KRR_CHECK_LAUNCH();
     }
     return KRR_OK;

@@ -363,9 +363,12 @@ int launch_kss(krr_ctx* ctx, const float* XS, int k, int d, double sigma, double
 // In-place lower Cholesky of the k x k row-major A (upper part ignored).  Sets *info
 // (host) to 0 or to 1 + the first column whose pivot is <= tau (or not finite); the
 // columns before it are final.
-int launch_potrf(krr_ctx* ctx, double* A, int k, int* info, double tau = 0.0);
-// Solve L X = B in place (B k x k row-major), L lower k x k row-major.
-int launch_trsm_lower(krr_ctx* ctx, const double* L, double* B, int k);
+// dinv (potrf_dinv) receives the inverses of L's diagonal blocks, for launch_tri_inverse.
+int potrf_dinv(krr_ctx* ctx, int k, double** dinv);
+int launch_potrf(krr_ctx* ctx, double* A, int k, int* info, double* dinv, double tau = 0.0);
+int launch_diag_inverse(krr_ctx* ctx, const double* L, int k, double* dinv);   // of any lower L
+// B (identity on entry) <- L^{-1}, k x k row-major, lower
+int launch_tri_inverse(krr_ctx* ctx, const double* L, const double* dinv, double* B, int k);
 int launch_transpose64(krr_ctx* ctx, const double* A, double* At, int k);
 int launch_to_float_transposed(krr_ctx* ctx, const double* A, int k, float* Out, int ldo);
 int launch_set_identity(krr_ctx* ctx, double* A, int k);

@@ -22,7 +22,6 @@ namespace krr {
 int qrcp_core(krr_ctx* ctx, float* Y, long long n, int l, int ldy, int k, int* piv, float* rdiag,
               const int* forced, float* Rout, double** nrm_out);
 int launch_set_identity(krr_ctx* ctx, double* A, int k);
-int launch_trsm_lower(krr_ctx* ctx, const double* L, double* B, int k);
 int launch_transpose64(krr_ctx* ctx, const double* A, double* At, int k);
 
 // R11[a][b] = R_a,piv[b] (upper triangular, FP64, row-major)
@@ -152,7 +151,10 @@ static int rrqr_measure(krr_ctx* ctx, const float* Rout, long long n, int k, con
     KRR_CHECK_LAUNCH();
     KRR_RET(launch_transpose64(ctx, R11, L, k));   // L = R11^T, lower
     KRR_RET(launch_set_identity(ctx, Linv, k));
-    KRR_RET(launch_trsm_lower(ctx, L, Linv, k));   // Linv = R11^{-T}
+    double* dinv;
+    KRR_RET(potrf_dinv(ctx, k, &dinv));
+    KRR_RET(launch_diag_inverse(ctx, L, k, dinv));
+    KRR_RET(launch_tri_inverse(ctx, L, dinv, Linv, k));   // Linv = R11^{-T}
     k_rrqr_w<<<k, 256, 0, ctx->stream>>>(Linv, k, W32, wn);
     KRR_CHECK_LAUNCH();
     k_rrqr_rho<<<grid, 256, 0, ctx->stream>>>(W32, k, Rout, n, nrm, wn, bval, bi, bj);
