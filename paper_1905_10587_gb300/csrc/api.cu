@@ -92,6 +92,7 @@ int buf(krr_ctx* ctx, const char* name, size_t bytes, void** out) {
 
 // launchers implemented in cg.cu that only the drivers use
 int cg_vec_blocks(krr_ctx* ctx);
+int apply_blocks(krr_ctx* ctx);
 int launch_cg_start(krr_ctx* ctx, const float* r, const float* z, int nrhs, double* rz_part,
                     double* rr_part);
 int launch_cg_alpha(krr_ctx* ctx, const float* p, const float* q, int nrhs, double* part);
@@ -761,8 +762,8 @@ int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol
     const double t0 = now_ms();
     const long long n = ctx->n;
     const long long tot = n * nrhs;
-    const int nb = cg_vec_blocks(ctx);
-    if (nb != cg64_vec_blocks(ctx)) return fail(ctx, KRR_E_STATE, "vector block counts differ");
+    // per-block partial sums of the vector kernels of either recurrence and of the apply
+    const int nb = std::max(std::max(cg_vec_blocks(ctx), cg64_vec_blocks(ctx)), apply_blocks(ctx));
     double *r64, *ynorm2, *rnorm2;
     float *x, *r, *z, *p, *q;
     double *part1, *part2, *part3;

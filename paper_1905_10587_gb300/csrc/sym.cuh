@@ -41,14 +41,14 @@ struct SyGrid {
 
 // Sums each a[m] over the lanes that differ in bit ST and the lower bits halved in turn, down to
 // N >> levels values: a lane keeps the half of the values its bit selects and sends the other.
-template <int N, int ST>
-__device__ __forceinline__ void lane_sum(float* a, int lane) {
+template <int N, int ST, class T>
+__device__ __forceinline__ void lane_sum(T* a, int lane) {
     constexpr int H = N / 2;
     const bool up = (lane & ST) != 0;
 #pragma unroll
     for (int m = 0; m < H; ++m) {
-        const float send = up ? a[m] : a[m + H];
-        const float keep = up ? a[m + H] : a[m];
+        const T send = up ? a[m] : a[m + H];
+        const T keep = up ? a[m + H] : a[m];
         a[m] = keep + __shfl_xor_sync(0xffffffffu, send, ST);
     }
     if constexpr (H > 1) lane_sum<H, ST / 2>(a, lane);

@@ -1021,6 +1021,7 @@ __global__ void k_pv_vscale(const float* __restrict__ V, int ldv, int n, int* __
     __shared__ float red[32];
     const int q = blockIdx.x;
     float m = 0.f;
+#pragma unroll 8
     for (int j = threadIdx.x; j < n; j += blockDim.x) m = fmaxf(m, fabsf(V[(size_t)q * ldv + j]));
     m = warp_max(m);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
@@ -1416,7 +1417,7 @@ static int launch_kmvm_tcpv(krr_ctx* ctx, const unsigned char* FA, long long nr,
     KRR_RET(bufT(ctx, "pv_vt", vbytes * (ncp / PV_BN), &Vt));
     KRR_RET(bufT(ctx, "pv_vexp", 16, &vexp));
     KRR_RET(bufT(ctx, "pv_vsc", 16, &vsc));
-    k_pv_vscale<<<nrhs, 512, 0, ctx->stream>>>(V, (int)nc, (int)nc, vexp, vsc);
+    k_pv_vscale<<<nrhs, 1024, 0, ctx->stream>>>(V, (int)nc, (int)nc, vexp, vsc);
     KRR_CHECK_LAUNCH();
     const long long nsplit = (long long)vrows * ncp;
     k_pv_vsplit<<<ceil_div(nsplit, 256), 256, 0, ctx->stream>>>(V, (int)nc, (int)nc, ncp, nrhs, vrows, vexp, Vt);
