@@ -152,6 +152,7 @@ template <int NQ, bool ONE>
 __global__ void __launch_bounds__(VT)
 k_gemv_t(const float* __restrict__ F, long long n, int ldF, const float* __restrict__ R,
          long long ldr, long long rows_per, int CW, float2* __restrict__ upart) {
+    pdl_entry();
     __shared__ float sr[NQ][GT_ROWS];
     __shared__ float2 red[ONE ? 1 : VT][4];
     const long long r0 = (long long)blockIdx.x * rows_per;
@@ -242,6 +243,7 @@ template <class T>
 __global__ void __launch_bounds__(256)
 k_gemv_t_reduce(const T* __restrict__ upart, int nblk, int nq, int k, int ldF,
                 double* __restrict__ u) {
+    pdl_entry();
     __shared__ double red[32][9];
     const int c = threadIdx.x & 7, g = threadIdx.x >> 3;
     const int a = blockIdx.x * 8 + c;
@@ -269,6 +271,7 @@ template <int NQ, int TPR>
 __global__ void __launch_bounds__(TG_T) k_tri_gemv(const double* __restrict__ T, int k,
                                                    const double* __restrict__ x, bool lower,
                                                    double* __restrict__ y) {
+    pdl_entry();
     __shared__ double red[NQ][TG_T / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int a = TPR == 32 ? blockIdx.x * (TG_T / 32) + w : (int)blockIdx.x;
@@ -316,9 +319,9 @@ static tri_fn tri_pick1(int nq) {
 int launch_tri_gemv(krr_ctx* ctx, const double* T, int k, const double* x, int nq, bool lower, double* y) {
     if (nq < 1 || nq > 8) return fail(ctx, KRR_E_INVAL, "triangular product: bad column count");
     if (k <= 512)
-        tri_pick1<32>(nq)<<<ceil_div(k, TG_T / 32), TG_T, 0, ctx->stream>>>(T, k, x, lower, y);
+        launch_pdl(tri_pick1<32>(nq), ceil_div(k, TG_T / 32), TG_T, 0, ctx->stream, T, k, x, lower, y);
     else
-        tri_pick1<TG_T>(nq)<<<k, TG_T, 0, ctx->stream>>>(T, k, x, lower, y);
+        launch_pdl(tri_pick1<TG_T>(nq), k, TG_T, 0, ctx->stream, T, k, x, lower, y);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -330,6 +333,7 @@ __global__ void __launch_bounds__(VT)
 k_gemv_n_apply(const float* __restrict__ F, long long n, int k, int ldF, const double* __restrict__ v,
                const float* __restrict__ R, long long ldr, float inv_beta, float* __restrict__ Z,
                double* __restrict__ rz_part, CGScalars* cg, int q0) {
+    pdl_entry();
     extern __shared__ float4 sv4[];   // NQ x ld4
     const int ld4 = ldF >> 2;
     for (int e = threadIdx.x; e < NQ * ld4; e += VT) {
@@ -455,9 +459,9 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
         const gemv_n_fn gn = gns[nq - 1];
         const float* Rq = R + (size_t)q0 * n;
         float* Zq = Z + (size_t)q0 * n;
-        gt<<<nt, VT, 0, ctx->stream>>>(ctx->F, n, ldF, Rq, n, rows_per, CW, upart);
+        launch_pdl_if(nt < 4 * ctx->num_sms, gt, nt, VT, 0, ctx->stream, ctx->F, n, ldF, Rq, n, rows_per, CW, upart);
         KRR_CHECK_LAUNCH();
-        k_gemv_t_reduce<<<dim3(ceil_div(k, 8), nq), 256, 0, ctx->stream>>>(upart, nt, nq, k, ldF, u);
+        launch_pdl(k_gemv_t_reduce<float2>, dim3(ceil_div(k, 8), nq), 256, 0, ctx->stream, upart, nt, nq, k, ldF, u);
         KRR_CHECK_LAUNCH();
         KRR_RET(launch_tri_gemv(ctx, ctx->T2, k, u, nq, true, u1));
         KRR_RET(launch_tri_gemv(ctx, ctx->T2t, k, u1, nq, false, v));
@@ -465,9 +469,8 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
         if (smem > 48 * 1024) {
             KRR_RET(allow_max_dynamic_smem(ctx, (const void*)gn));
         }
-        gn<<<nb, VT, smem, ctx->stream>>>(ctx->F, n, k, ldF, v, Rq, n, inv_beta, Zq,
-                                          rz_part ? rz_part + (size_t)q0 * nb : nullptr,
-                                          rz_part && with_beta ? ctx->cg : nullptr, q0);
+        launch_pdl_if(nb < 4 * ctx->num_sms, gn, nb, VT, smem, ctx->stream, ctx->F, n, k, ldF, v, Rq, n, inv_beta, Zq,
+                   rz_part ? rz_part + (size_t)q0 * nb : nullptr, rz_part && with_beta ? ctx->cg : nullptr, q0);
         KRR_CHECK_LAUNCH();
     }
     return KRR_OK;
@@ -500,6 +503,7 @@ __global__ void k_cg_alpha(CGScalars* cg, const double* __restrict__ part, int n
 __global__ void __launch_bounds__(VT)
 k_cg_dot_alpha(const float* __restrict__ p, const float* __restrict__ qv, long long n, CGScalars* cg,
                double* __restrict__ part) {
+    pdl_entry();
     {
         const int q = blockIdx.y;
         double s = 0.0;
@@ -543,6 +547,7 @@ __global__ void __launch_bounds__(VT)
 k_cg_update_xr(float* __restrict__ x, float* __restrict__ r, const float* __restrict__ p,
                const float* __restrict__ qv, long long n, CGScalars* cg,
                double* __restrict__ part, double tol2) {
+    pdl_entry();
     {
         const int q = blockIdx.y;
         const float a = (float)cg->a[q];
@@ -582,6 +587,7 @@ __global__ void k_cg_beta(CGScalars* cg, const double* __restrict__ part, int nb
 // p = z + b p; with_beta (b came with the apply): rz = rz_new, which nothing here reads
 __global__ void __launch_bounds__(VT)
 k_cg_update_p(float* __restrict__ p, const float* __restrict__ z, long long n, CGScalars* cg, bool with_beta) {
+    pdl_entry();
     const int q = blockIdx.y;
     if (with_beta && blockIdx.x == 0 && threadIdx.x == 0) cg->rz[q] = cg->rz_new[q];
     const float b = (float)cg->b[q];
@@ -650,7 +656,7 @@ int launch_cg_start(krr_ctx* ctx, const float* r, const float* z, int nrhs, doub
 
 int launch_cg_alpha(krr_ctx* ctx, const float* p, const float* q, int nrhs, double* part) {
     const int nb = vec_blocks(ctx, ctx->n);
-    k_cg_dot_alpha<<<dim3(nb, nrhs), VT, 0, ctx->stream>>>(p, q, ctx->n, ctx->cg, part);
+    launch_pdl(k_cg_dot_alpha, dim3(nb, nrhs), VT, 0, ctx->stream, p, q, ctx->n, ctx->cg, part);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -658,7 +664,7 @@ int launch_cg_alpha(krr_ctx* ctx, const float* p, const float* q, int nrhs, doub
 int launch_cg_update_xr(krr_ctx* ctx, float* x, float* r, const float* p, const float* q, int nrhs,
                         double* part, double tol2) {
     const int nb = vec_blocks(ctx, ctx->n);
-    k_cg_update_xr<<<dim3(nb, nrhs), VT, 0, ctx->stream>>>(x, r, p, q, ctx->n, ctx->cg, part, tol2);
+    launch_pdl(k_cg_update_xr, dim3(nb, nrhs), VT, 0, ctx->stream, x, r, p, q, ctx->n, ctx->cg, part, tol2);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -669,7 +675,7 @@ int launch_cg_beta_p(krr_ctx* ctx, float* p, const float* z, int nrhs, const dou
         k_cg_beta<<<1, 32 * nrhs, 0, ctx->stream>>>(ctx->cg, rz_part, rz_blocks(ctx), nrhs);
         KRR_CHECK_LAUNCH();
     }
-    k_cg_update_p<<<dim3(nb, nrhs), VT, 0, ctx->stream>>>(p, z, ctx->n, ctx->cg, with_beta);
+    launch_pdl(k_cg_update_p, dim3(nb, nrhs), VT, 0, ctx->stream, p, z, ctx->n, ctx->cg, with_beta);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -699,7 +705,7 @@ int launch_identity_apply64(krr_ctx* ctx, const double* R, int nrhs, double* Z, 
 
 // pieces used by the FP64 recurrence (cg64.cu)
 int launch_gemv_t_reduce(krr_ctx* ctx, const double* upart, int nblk, int nq, int k, int ldF, double* u) {
-    k_gemv_t_reduce<<<dim3(ceil_div(k, 8), nq), 256, 0, ctx->stream>>>(upart, nblk, nq, k, ldF, u);
+    launch_pdl(k_gemv_t_reduce<double>, dim3(ceil_div(k, 8), nq), 256, 0, ctx->stream, upart, nblk, nq, k, ldF, u);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }

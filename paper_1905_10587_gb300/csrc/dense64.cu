@@ -62,6 +62,7 @@ constexpr int PF_Y = 8;
 __global__ void __launch_bounds__(NB * PF_Y)
 k_potf2(double* __restrict__ A, int k, int j0, int nb, double tau, int* __restrict__ info,
         double* __restrict__ Linv) {
+    pdl_entry();
     __shared__ double s[NB][NB + 1], ei[NB][NB + 1], w[NB], sd[NB];
     const int c = threadIdx.x, y = threadIdx.y;
 #pragma unroll
@@ -107,6 +108,7 @@ k_potf2(double* __restrict__ A, int k, int j0, int nb, double tau, int* __restri
 // (a warp per row: its inputs are read by the warp before any of its outputs is written)
 __global__ void __launch_bounds__(128)
 k_potrf_panel(double* __restrict__ A, int k, int j0, int nb, const double* __restrict__ Linv) {
+    pdl_entry();
     __shared__ double L[NB][NB + 1];
     __shared__ double x[4][NB];
     for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) L[e / NB][e % NB] = Linv[e];
@@ -127,6 +129,7 @@ k_potrf_panel(double* __restrict__ A, int k, int j0, int nb, const double* __res
 constexpr int DT = 16;
 __global__ void __launch_bounds__(DT * DT)
 k_potrf_update(double* __restrict__ A, int k, int j0, int nb, int t0) {
+    pdl_entry();
     // blockIdx.x enumerates the lower-triangular tile pairs of the trailing matrix
     const int p = blockIdx.x;
     int bi = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
@@ -171,14 +174,14 @@ int launch_potrf(krr_ctx* ctx, double* A, int k, int* info_host, double* dinv, d
     for (int j0 = 0; j0 < k; j0 += NB) {
         const int nb = std::min(NB, k - j0);
         double* Lj = dinv + (size_t)(j0 / NB) * NB * NB;
-        k_potf2<<<1, dim3(NB, PF_Y), 0, ctx->stream>>>(A, k, j0, nb, tau, info, Lj);
+        launch_pdl(k_potf2, 1, dim3(NB, PF_Y), 0, ctx->stream, A, k, j0, nb, tau, info, Lj);
         KRR_CHECK_LAUNCH();
         const int rest = k - j0 - nb;
         if (rest <= 0) break;
-        k_potrf_panel<<<ceil_div(rest, 4), 128, 0, ctx->stream>>>(A, k, j0, nb, Lj);
+        launch_pdl(k_potrf_panel, ceil_div(rest, 4), 128, 0, ctx->stream, A, k, j0, nb, Lj);
         KRR_CHECK_LAUNCH();
         const int tb = (rest + DT - 1) / DT;
-        k_potrf_update<<<tb * (tb + 1) / 2, DT * DT, 0, ctx->stream>>>(A, k, j0, nb, j0 + nb);
+        launch_pdl(k_potrf_update, tb * (tb + 1) / 2, DT * DT, 0, ctx->stream, A, k, j0, nb, j0 + nb);
         KRR_CHECK_LAUNCH();
     }
     k_zero_upper<<<ceil_div((long long)k * k, 256), 256, 0, ctx->stream>>>(A, k);
@@ -199,6 +202,7 @@ int potrf_dinv(krr_ctx* ctx, int k, double** dinv) {
 constexpr int TD_C = 8;
 __global__ void __launch_bounds__(NB * TD_C)
 k_trinv_diag(const double* __restrict__ Linv, double* __restrict__ B, int k, int j0, int nb, int ncols) {
+    pdl_entry();
     __shared__ double sl[NB][NB + 1];
     __shared__ double sx[NB][TD_C + 1];
     for (int e = threadIdx.x; e < NB * NB; e += NB * TD_C) sl[e / NB][e % NB] = Linv[e];
@@ -219,6 +223,7 @@ k_trinv_diag(const double* __restrict__ Linv, double* __restrict__ B, int k, int
 // B[i, c] -= sum_m L[i, j0+m] B[j0+m, c]  for i >= j0+nb, c < ncols, in 16 x 16 tiles
 __global__ void __launch_bounds__(DT * DT)
 k_trinv_update(const double* __restrict__ L, double* __restrict__ B, int k, int j0, int nb, int ncols) {
+    pdl_entry();
     __shared__ double sl[DT][NB + 1];
     __shared__ double sx[NB][DT + 1];
     const int r0 = j0 + nb + blockIdx.y * DT, c0 = blockIdx.x * DT;
@@ -272,13 +277,13 @@ int launch_tri_inverse(krr_ctx* ctx, const double* L, const double* dinv, double
     for (int j0 = 0; j0 < k; j0 += NB) {
         const int nb = std::min(NB, k - j0);
         const int ncols = j0 + nb;   // columns >= j0 + nb are still zero in these rows
-        k_trinv_diag<<<ceil_div(ncols, TD_C), NB * TD_C, 0, ctx->stream>>>(dinv + (size_t)(j0 / NB) * NB * NB, B, k,
-                                                                           j0, nb, ncols);
+        launch_pdl(k_trinv_diag, ceil_div(ncols, TD_C), NB * TD_C, 0, ctx->stream,
+                   dinv + (size_t)(j0 / NB) * NB * NB, B, k, j0, nb, ncols);
         KRR_CHECK_LAUNCH();
         const int rest = k - j0 - nb;
         if (rest <= 0) break;
         dim3 grid(ceil_div(ncols, DT), ceil_div(rest, DT));
-        k_trinv_update<<<grid, DT * DT, 0, ctx->stream>>>(L, B, k, j0, nb, ncols);
+        launch_pdl(k_trinv_update, grid, DT * DT, 0, ctx->stream, L, B, k, j0, nb, ncols);
         KRR_CHECK_LAUNCH();
     }
     return KRR_OK;

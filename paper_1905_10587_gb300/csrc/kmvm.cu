@@ -497,6 +497,7 @@ k_kmvm2(const float* __restrict__ Pr, int nr, const float* __restrict__ Pc, int 
 __global__ void k_kmvm_reduce(const double* __restrict__ part, int splits, int nr, int nrhs,
                               const float* __restrict__ V, int ldv, float beta,
                               float* __restrict__ Q, int ldq, double ksc) {
+    pdl_entry();
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (long long)nr * nrhs) return;
     const int q = (int)(e / nr);
@@ -519,8 +520,8 @@ double ex2_bias_scale(const krr_ctx* ctx) {
 int launch_kmvm_reduce(krr_ctx* ctx, const double* part, int splits, int nr, int nrhs, const float* V,
                        int ldv, float beta, float* Q, int ldq) {
     const long long tot = (long long)nr * nrhs;
-    k_kmvm_reduce<<<ceil_div(tot, 256), 256, 0, ctx->stream>>>(part, splits, nr, nrhs, V, ldv, beta, Q,
-                                                                ldq, ex2_bias_scale(ctx));
+    launch_pdl(k_kmvm_reduce, ceil_div(tot, 256), 256, 0, ctx->stream, part, splits, nr, nrhs, V, ldv, beta, Q, ldq,
+               ex2_bias_scale(ctx));
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -708,9 +709,8 @@ int launch_kmvm(krr_ctx* ctx, const float* Pr, long long nr, const float* Pc, lo
                                          (double)beta, Q64 + (size_t)(done / 2) * nr, ksc));
         } else if (part) {
             const long long tot = nr * chunk;
-            k_kmvm_reduce<<<ceil_div(tot, 256), 256, 0, ctx->stream>>>(part, splits, (int)nr, chunk,
-                                                                        Vc, (int)nc, beta, Qc,
-                                                                        (int)nr, ksc);
+            launch_pdl(k_kmvm_reduce, ceil_div(tot, 256), 256, 0, ctx->stream, part, splits, (int)nr, chunk, Vc,
+                       (int)nc, beta, Qc, (int)nr, ksc);
             KRR_CHECK_LAUNCH();
         }
         done += chunk;
@@ -897,9 +897,8 @@ int kmvm_into_scratch(cudaStream_t stream, int num_sms, const float* Xr, long lo
                                                           (float)beta, 0.f, 0.f, Qc, (int)nr,
                                                           splits > 1 ? part : nullptr);
         if (splits > 1)
-            k_kmvm_reduce<<<ceil_div(nr * chunk, 256), 256, 0, stream>>>(part, splits, (int)nr, chunk,
-                                                                          Vc, (int)nc, (float)beta,
-                                                                          Qc, (int)nr, 1.0);
+            launch_pdl(k_kmvm_reduce, ceil_div(nr * chunk, 256), 256, 0, stream, part, splits, (int)nr, chunk, Vc,
+                       (int)nc, (float)beta, Qc, (int)nr, 1.0);
         done += chunk;
     }
     return cudaGetLastError() == cudaSuccess ? KRR_OK : KRR_E_CUDA;

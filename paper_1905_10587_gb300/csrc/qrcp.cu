@@ -114,6 +114,7 @@ __device__ __forceinline__ void qr_block_key(unsigned long long best, unsigned l
 __global__ void __launch_bounds__(QR_THREADS)
 k_qr_norms(const float* __restrict__ Y, long long n, int l, int ldy, double* __restrict__ nrm,
            unsigned long long* __restrict__ bkeys) {
+    pdl_entry();
     const int lane = threadIdx.x & 31;
     const long long w0 = (long long)blockIdx.x * QR_WARPS + (threadIdx.x >> 5);
     const long long nw = (long long)gridDim.x * QR_WARPS;
@@ -156,6 +157,7 @@ k_qr_reflector(const float* __restrict__ Y, long long n, int l, int ldy, int m, 
                double* __restrict__ nrm, const unsigned long long* __restrict__ bkeys, int nbk,
                int* __restrict__ piv, float* __restrict__ rdiag, const int* __restrict__ forced,
                float* __restrict__ Rout) {
+    pdl_entry();
     extern __shared__ float2 zs[];   // z in pairs, by coordinate
     __shared__ double red[QR_REF_WARPS];
     __shared__ float2 redf[QR_REF_WARPS];
@@ -316,6 +318,7 @@ k_qr_step(const float* __restrict__ Y, long long n, int l, int ldy, int m, int j
           float* __restrict__ C, const float* __restrict__ Vp, const float* __restrict__ tau,
           const float* __restrict__ g, double* __restrict__ nrm, unsigned long long* __restrict__ bkeys,
           float* __restrict__ Rout) {
+    pdl_entry();
     constexpr int S = U == 8 ? 0 : U == 4 ? 1 : U == 2 ? 2 : 3;   // value q of row u: in lane (4 u + q) 2^S
     extern __shared__ float qsm[];    // v_m[m:] zero-padded, then the warps' rings
     __shared__ float gsh[QH_B], vjm[QH_B];
@@ -442,6 +445,7 @@ __host__ __device__ inline size_t qp_smem(int nb, int L) {
 __global__ void __launch_bounds__(QP_THREADS, 1)
 k_qr_panel(float* __restrict__ Y, long long n, int l, int ldy, int m1, int nb, const float* __restrict__ C,
            const float* __restrict__ Vp, double* __restrict__ nrm, unsigned long long* __restrict__ bkeys) {
+    pdl_entry();
     extern __shared__ __align__(16) float qps[];   // the warps' coefficients, then nb x L reflectors
     const int L = l - m1;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -551,9 +555,8 @@ int qrcp_core(krr_ctx* ctx, float* Y, long long n, int l, int ldy, int k, int* p
         for (int jm = 0; jm < nb; ++jm) {
             const int m = m0 + jm;
             const int L = l - m;
-            k_qr_reflector<<<1, ref_threads, sizeof(float2) * l, ctx->stream>>>(Y, n, l, ldy, m, jm, C, Vp, tau, g,
-                                                                               nrm, bkeys, nbk, piv, rdiag, forced,
-                                                                               Rout);
+            launch_pdl(k_qr_reflector, 1, ref_threads, sizeof(float2) * l, ctx->stream, Y, n, l, ldy, m, jm, C, Vp,
+                       tau, g, nrm, bkeys, nbk, piv, rdiag, forced, Rout);
             KRR_CHECK_LAUNCH();
             if (m + 1 < k || Rout) {
                 const int kp = (L + 31) / 32;
@@ -564,8 +567,8 @@ int qrcp_core(krr_ctx* ctx, float* Y, long long n, int l, int ldy, int k, int* p
                 const int per_sm = std::max(1, std::min(QR_STEP_BLOCKS, (int)(220 * 1024 / smem)));
                 const int rw = (int)ceil_div(n, (long long)ctx->num_sms * per_sm * QR_WARPS * st.U) * st.U;
                 nbk = (int)ceil_div(n, (long long)QR_WARPS * rw);
-                st.fn<<<nbk, QR_THREADS, smem, ctx->stream>>>(Y, n, l, ldy, m, jm, rw, kp, C, Vp, tau, g, nrm, bkeys,
-                                                              Rout);
+                launch_pdl(st.fn, nbk, QR_THREADS, smem, ctx->stream, Y, n, l, ldy, m, jm, rw, kp, C, Vp, tau, g,
+                           nrm, bkeys, Rout);
                 KRR_CHECK_LAUNCH();
             }
         }
@@ -574,7 +577,8 @@ int qrcp_core(krr_ctx* ctx, float* Y, long long n, int l, int ldy, int k, int* p
             // the panel's updates reach the coordinates beyond it; the exact norms replace
             // the downdated ones and give the next pivot
             nbk = (int)std::min<long long>(ctx->num_sms, ceil_div(n, QP_R));
-            k_qr_panel<<<nbk, QP_THREADS, qp_smem(nb, l - m1), ctx->stream>>>(Y, n, l, ldy, m1, nb, C, Vp, nrm, bkeys);
+            launch_pdl(k_qr_panel, nbk, QP_THREADS, qp_smem(nb, l - m1), ctx->stream, Y, n, l, ldy, m1, nb, C, Vp,
+                       nrm, bkeys);
             KRR_CHECK_LAUNCH();
         }
     }

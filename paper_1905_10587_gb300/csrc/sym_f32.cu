@@ -58,6 +58,7 @@ template <int D, int R, bool RAW>
 __global__ void __launch_bounds__(SF_ROWS / R * 4)
 k_sym_f32(const float* __restrict__ P, SyGrid sg, const float* __restrict__ V, float nsc,
           float2* __restrict__ rowpart, float2* __restrict__ colpart) {
+    pdl_entry();
     constexpr int NT = SF_ROWS / R * 4;            // threads
     constexpr int NW = NT / 32;
     constexpr int PS = (D + 1 + 3) / 4 * 4;
@@ -278,7 +279,7 @@ int launch_kmvm_sym_f32(krr_ctx* ctx, const float* P, long long n, int d, float 
     float2 *rowpart, *colpart;
     KRR_RET(bufT(ctx, "sy_row", (size_t)(g.G + g.nblk) * g.rows(), &rowpart));
     KRR_RET(bufT(ctx, "sy_col", (size_t)g.col_base(g.NU), &colpart));
-    fn<<<g.G, threads, 0, ctx->stream>>>(P, g, V, raw_nsc, rowpart, colpart);
+    launch_pdl(fn, g.G, threads, 0, ctx->stream, P, g, V, raw_nsc, rowpart, colpart);
     KRR_CHECK_LAUNCH();
     return launch_sym_reduce(ctx, g, rowpart, colpart, V, beta, 1.0, nullptr, Q);
 }

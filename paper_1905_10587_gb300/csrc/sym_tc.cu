@@ -65,6 +65,7 @@ __device__ __forceinline__ void sy_bar(int id, int threads) {
 constexpr int SY_PAD = 1024;
 __global__ void __launch_bounds__(SY_PAD) k_sym_pad(const float* __restrict__ V, int n, int np,
                                                     float* __restrict__ Vp, float* __restrict__ bmax) {
+    pdl_entry();
     __shared__ float red[SY_PAD / 32];
     const int i = blockIdx.x * SY_PAD + threadIdx.x;
     const float v = i < n ? V[i] : 0.f;
@@ -92,6 +93,7 @@ k_kmvm_sym(const unsigned char* __restrict__ FA, const unsigned char* __restrict
            const float* __restrict__ Vp, float2* __restrict__ rowpart, float2* __restrict__ colpart,
            const float* __restrict__ bmax, int nbmax, double* __restrict__ vscale, int* __restrict__ err,
            long long wlimit, int stall_copies) {
+    pdl_entry();
     constexpr int NBUF = 512 / BN;                     // TMEM buffers
     constexpr int CT = BN / SY_T;                      // feature tiles per column unit
     constexpr int CW = BN / 2;                         // columns per epilogue warp
@@ -469,6 +471,7 @@ __global__ void __launch_bounds__(SY_T * SYR_G)
 k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __restrict__ colpart,
              const float* __restrict__ V, float beta, double ksc, const double* __restrict__ vscale,
              float* __restrict__ Q) {
+    pdl_entry();
     __shared__ double red[SYR_G][SY_T];
     const int x = threadIdx.x & (SY_T - 1), grp = threadIdx.x / SY_T;
     const int i = blockIdx.x * SY_T + x;
@@ -499,7 +502,8 @@ k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __rest
 
 int launch_sym_reduce(krr_ctx* ctx, const SyGrid& g, const float2* rowpart, const float2* colpart, const float* V,
                       float beta, double ksc, const double* vscale, float* Q) {
-    k_sym_reduce<<<g.NU * g.BN / SY_T, SY_T * SYR_G, 0, ctx->stream>>>(g, rowpart, colpart, V, beta, ksc, vscale, Q);
+    launch_pdl(k_sym_reduce, g.NU * g.BN / SY_T, SY_T * SYR_G, 0, ctx->stream, g, rowpart, colpart, V, beta, ksc,
+               vscale, Q);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -579,11 +583,11 @@ int launch_kmvm_sym(krr_ctx* ctx, const unsigned char* FA, const unsigned char* 
     KRR_RET(allow_max_dynamic_smem(ctx, (const void*)fn));
     const long long wlimit = ctx->opts.wait_limit_log2 > 0 ? (1LL << ctx->opts.wait_limit_log2)
                                                            : kWaitLimitDefault;
-    k_sym_pad<<<nbmax, SY_PAD, 0, ctx->stream>>>(V, (int)n, np, Vp, bmax);
+    launch_pdl(k_sym_pad, nbmax, SY_PAD, 0, ctx->stream, V, (int)n, np, Vp, bmax);
     KRR_CHECK_LAUNCH();
     const size_t smem = std::max<size_t>(sym_smem(Kp, BN, RU), 120 * 1024);   // one CTA per SM (TMEM)
-    fn<<<g.G, SY_THREADS, smem, ctx->stream>>>(FA, FB, Kp, g, Vp, rowpart, colpart, bmax, nbmax, vscale, err,
-                                               wlimit, ctx->opts.test_stall_copies);
+    launch_pdl(fn, g.G, SY_THREADS, smem, ctx->stream, FA, FB, Kp, g, Vp, rowpart, colpart, bmax, nbmax, vscale,
+               err, wlimit, ctx->opts.test_stall_copies);
     KRR_CHECK_LAUNCH();
     return launch_sym_reduce(ctx, g, rowpart, colpart, V, beta, ex2_bias_scale(ctx), vscale, Q);
 }

@@ -220,6 +220,7 @@ constexpr int VF_BLK = 1024;   // columns per block of the partition
 // floats order like their bits, so atomicMax on the bits is exact; *vmax starts at 0)
 __global__ void __launch_bounds__(VF_BLK) k_vf_count(const float* __restrict__ V, int n, int* __restrict__ cnt,
                                                       unsigned* __restrict__ vmax) {
+    pdl_entry();
     __shared__ int wc[VF_BLK / 32];
     __shared__ unsigned wm[VF_BLK / 32];
     const int j = blockIdx.x * VF_BLK + threadIdx.x;
@@ -250,6 +251,7 @@ __global__ void __launch_bounds__(VF_BLK) k_vf_count(const float* __restrict__ V
 // nblk <= 2^20 / 1024)
 __global__ void k_vf_scan(const int* __restrict__ cnt, int nblk, int* __restrict__ off, int* __restrict__ bnd,
                           const unsigned* __restrict__ vmax, int* __restrict__ vexp, double* __restrict__ vsc) {
+    pdl_entry();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     int t = 0;
     for (int b = 0; b < nblk; ++b) {
@@ -273,6 +275,7 @@ __global__ void __launch_bounds__(VF_BLK)
 k_vf_scatter(const float* __restrict__ V, int n, int ncp, const int* __restrict__ off, const int* __restrict__ bnd,
              const int* __restrict__ vexp, const unsigned char* __restrict__ FB, int Kp, int k0,
              unsigned char* __restrict__ FBv) {
+    pdl_entry();
     __shared__ int wpre[VF_BLK / 32];
     const int j = blockIdx.x * VF_BLK + threadIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -359,6 +362,7 @@ k_kmvm_tc(const unsigned char* __restrict__ FA, const unsigned char* __restrict_
           int nr, int nc, int ncp, const float* __restrict__ Vp, int items, int splits,
           int tiles_per_split, int ns, double* __restrict__ part, int* __restrict__ err,
           long long wlimit, int stall_copies, const int* __restrict__ vf_bnd, const double* __restrict__ vf_sc) {
+    pdl_entry();
     static_assert(!VF || NRHS == 1, "the V-folded form takes one right-hand side");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // swizzle atoms need 1024-byte alignment; the launch adds 1 KB of slack for this
@@ -737,6 +741,7 @@ template <int NRHS>
 __global__ void __launch_bounds__(PV_THREADS, 1)
 k_kmvm_tcpv(const __grid_constant__ PvWork w, int items, int* __restrict__ err, long long wlimit,
             int stall_copies) {
+    pdl_entry();
     static_assert(NRHS == 1 || NRHS == 2 || NRHS == 4 || NRHS == 8 || NRHS == 16, "right-hand sides");
     constexpr uint32_t VROWS = 2 * NRHS < 16 ? 16 : 2 * NRHS;   // Vh rows, Vl rows, zero rows
     constexpr uint32_t VSLAB = VROWS * 128u;          // bytes of 64 K of the V tile
@@ -1018,6 +1023,7 @@ k_kmvm_tcpv(const __grid_constant__ PvWork w, int items, int* __restrict__ err, 
 // not finite); vexp[q] = e_q and vsc[q] = 2^-(15 + e_q), the factor that undoes both scales.
 __global__ void k_pv_vscale(const float* __restrict__ V, int ldv, int n, int* __restrict__ vexp,
                             double* __restrict__ vsc) {
+    pdl_entry();
     __shared__ float red[32];
     const int q = blockIdx.x;
     float m = 0.f;
@@ -1045,6 +1051,7 @@ __global__ void k_pv_vscale(const float* __restrict__ V, int ldv, int n, int* __
 // K-major layout, zero beyond n.  One thread per (row, column).
 __global__ void k_pv_vsplit(const float* __restrict__ V, int ldv, int n, int ncp, int nrhs, int rows,
                             const int* __restrict__ vexp, unsigned char* __restrict__ Vt) {
+    pdl_entry();
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (long long)rows * ncp) return;
     const int r = (int)(e / ncp), j = (int)(e - (long long)r * ncp);
@@ -1324,6 +1331,7 @@ typedef void (*tc_fn)(const unsigned char*, const unsigned char*, int, int, int,
 // ---- grouped form: the same kernels over the problems of a batch, one launch each
 // Per (problem, right-hand side) block: the column's scale exponent, as k_pv_vscale.
 __global__ void k_pv_vscale_g(const PvPrep* __restrict__ tab, int nrhs) {
+    pdl_entry();
     __shared__ float red[32];
     const PvPrep& pp = tab[blockIdx.x / nrhs];
     const int q = blockIdx.x % nrhs;
@@ -1348,6 +1356,7 @@ __global__ void k_pv_vscale_g(const PvPrep* __restrict__ tab, int nrhs) {
 
 // The split of every problem's V into its tiles, as k_pv_vsplit; blocks blk0 .. of problem p.
 __global__ void k_pv_vsplit_g(const PvPrep* __restrict__ tab, int nprob, int nrhs, int rows) {
+    pdl_entry();
     int lo = 0, hi = nprob - 1;   // last problem whose first block is <= blockIdx.x
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -1372,9 +1381,9 @@ __global__ void k_pv_vsplit_g(const PvPrep* __restrict__ tab, int nprob, int nrh
 int pv_tile_bytes(int nrhs) { return std::max(16, 2 * nrhs) * PV_BN * 2; }
 
 int launch_pv_prep_grouped(krr_ctx* ctx, const PvPrep* tab_dev, int nprob, int nblk, int nrhs) {
-    k_pv_vscale_g<<<nprob * nrhs, 512, 0, ctx->stream>>>(tab_dev, nrhs);
+    launch_pdl(k_pv_vscale_g, nprob * nrhs, 512, 0, ctx->stream, tab_dev, nrhs);
     KRR_CHECK_LAUNCH();
-    k_pv_vsplit_g<<<nblk, 256, 0, ctx->stream>>>(tab_dev, nprob, nrhs, std::max(16, 2 * nrhs));
+    launch_pdl(k_pv_vsplit_g, nblk, 256, 0, ctx->stream, tab_dev, nprob, nrhs, std::max(16, 2 * nrhs));
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -1400,7 +1409,8 @@ int launch_kmvm_tcpv_table(krr_ctx* ctx, const PvProb* table_dev, int nprob, int
     w.table = table_dev;
     w.nprob = nprob;
     const int grid = std::min(items, ctx->num_sms);
-    fn<<<grid, PV_THREADS, pv_smem_bytes(nrhs), ctx->stream>>>(w, items, err, wlimit, ctx->opts.test_stall_copies);
+    launch_pdl(fn, grid, PV_THREADS, pv_smem_bytes(nrhs), ctx->stream, w, items, err, wlimit,
+               ctx->opts.test_stall_copies);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
@@ -1417,10 +1427,11 @@ static int launch_kmvm_tcpv(krr_ctx* ctx, const unsigned char* FA, long long nr,
     KRR_RET(bufT(ctx, "pv_vt", vbytes * (ncp / PV_BN), &Vt));
     KRR_RET(bufT(ctx, "pv_vexp", 16, &vexp));
     KRR_RET(bufT(ctx, "pv_vsc", 16, &vsc));
-    k_pv_vscale<<<nrhs, 1024, 0, ctx->stream>>>(V, (int)nc, (int)nc, vexp, vsc);
+    launch_pdl(k_pv_vscale, nrhs, 1024, 0, ctx->stream, V, (int)nc, (int)nc, vexp, vsc);
     KRR_CHECK_LAUNCH();
     const long long nsplit = (long long)vrows * ncp;
-    k_pv_vsplit<<<ceil_div(nsplit, 256), 256, 0, ctx->stream>>>(V, (int)nc, (int)nc, ncp, nrhs, vrows, vexp, Vt);
+    launch_pdl(k_pv_vsplit, ceil_div(nsplit, 256), 256, 0, ctx->stream, V, (int)nc, (int)nc, ncp, nrhs, vrows, vexp,
+               Vt);
     KRR_CHECK_LAUNCH();
     if (Kp != 64) return fail(ctx, KRR_E_INVAL, "P.V on tensor cores needs d <= 9");
     auto fn = nrhs == 16 ? &k_kmvm_tcpv<16> : nrhs == 8 ? &k_kmvm_tcpv<8> : nrhs == 4 ? &k_kmvm_tcpv<4>
@@ -1457,7 +1468,8 @@ static int launch_kmvm_tcpv(krr_ctx* ctx, const unsigned char* FA, long long nr,
     w.table = nullptr;
     w.nprob = 1;
     w.one = PvProb{FA, FB, Vt, vsc, part, (int)nr, (int)nc, Kp, splits, tps, items, 0, 0};
-    fn<<<grid, PV_THREADS, pv_smem_bytes(nrhs), ctx->stream>>>(w, items, err, wlimit, ctx->opts.test_stall_copies);
+    launch_pdl(fn, grid, PV_THREADS, pv_smem_bytes(nrhs), ctx->stream, w, items, err, wlimit,
+               ctx->opts.test_stall_copies);
     KRR_CHECK_LAUNCH();
     return launch_kmvm_reduce(ctx, part, splits, (int)nr, nrhs, V, (int)nc, beta, Q, (int)nr);
 }
@@ -1534,12 +1546,12 @@ int launch_kmvm_tc(krr_ctx* ctx, const unsigned char* FA, long long nr, const un
             KRR_RET(bufT(ctx, "vf_max", 1, &vmax));
             const float* Vc = V + (size_t)done * nc;
             KRR_TRY_CUDA(cudaMemsetAsync(vmax, 0, sizeof(unsigned), ctx->stream));
-            k_vf_count<<<nblk, VF_BLK, 0, ctx->stream>>>(Vc, (int)nc, cnt, vmax);
+            launch_pdl(k_vf_count, nblk, VF_BLK, 0, ctx->stream, Vc, (int)nc, cnt, vmax);
             KRR_CHECK_LAUNCH();
-            k_vf_scan<<<1, 32, 0, ctx->stream>>>(cnt, nblk, off, vf_bnd, vmax, vexp, vf_sc);
+            launch_pdl(k_vf_scan, 1, 32, 0, ctx->stream, cnt, nblk, off, vf_bnd, vmax, vexp, vf_sc);
             KRR_CHECK_LAUNCH();
-            k_vf_scatter<<<(unsigned)ceil_div(ncp, VF_BLK), VF_BLK, 0, ctx->stream>>>(
-                Vc, (int)nc, ncp, off, vf_bnd, vexp, FB, Kp, 6 * kernel_dim(d) + 6, FBv);
+            launch_pdl(k_vf_scatter, (unsigned)ceil_div(ncp, VF_BLK), VF_BLK, 0, ctx->stream, Vc, (int)nc, ncp, off,
+                       vf_bnd, vexp, FB, Kp, 6 * kernel_dim(d) + 6, FBv);
             KRR_CHECK_LAUNCH();
             FBk = FBv;
         } else {
@@ -1583,9 +1595,8 @@ int launch_kmvm_tc(krr_ctx* ctx, const unsigned char* FA, long long nr, const un
         const int grid = std::min(items, ctx->num_sms);
         const long long wlimit = ctx->opts.wait_limit_log2 > 0 ? (1LL << ctx->opts.wait_limit_log2)
                                                                : kWaitLimitDefault;
-        fn<<<grid, tc_threads(ew), smem_launch, ctx->stream>>>(FA, FBk, Kp, (int)nr, (int)nc, ncp, Vp, items,
-                                                               splits, tps, ns, part, err, wlimit,
-                                                               ctx->opts.test_stall_copies, vf_bnd, vf_sc);
+        launch_pdl(fn, grid, tc_threads(ew), smem_launch, ctx->stream, FA, FBk, Kp, (int)nr, (int)nc, ncp, Vp,
+                   items, splits, tps, ns, part, err, wlimit, ctx->opts.test_stall_copies, vf_bnd, vf_sc);
         KRR_CHECK_LAUNCH();
         // column groups (tile parity x column part) per split: ngroups * splits partial sums
         if (hp)
