@@ -97,7 +97,8 @@ int launch_cg_start(krr_ctx* ctx, const float* r, const float* z, int nrhs, doub
                     double* rr_part);
 int launch_cg_alpha(krr_ctx* ctx, const float* p, const float* q, int nrhs, double* part);
 int launch_cg_update_xr(krr_ctx* ctx, float* x, float* r, const float* p, const float* q, int nrhs,
-                        double* part, double tol2);
+                        double* part, double tol2,
+                        bool mirror, const int* tc_err);
 int launch_cg_beta_p(krr_ctx* ctx, float* p, const float* z, int nrhs, const double* rz_part, bool with_beta);
 int launch_cg_set_active(krr_ctx* ctx, const int* act_host, int nrhs);
 int launch_identity_apply(krr_ctx* ctx, const float* R, int nrhs, float* Z, double* rz_part);
@@ -751,6 +752,24 @@ static int square_product64(krr_ctx* ctx, const double* p64, int nrhs, float* ps
                        nullptr, 0.f, p64, q64);
 }
 
+// Until the scalar mirror shows the last update of x and r queued; the stream's state is asked now and
+// then, so that an error in what was queued ends the wait.
+static int wait_mirror(krr_ctx* ctx) {
+    const unsigned long long* seq = &ctx->cg_host->seq;
+    auto there = [&]() { return __atomic_load_n(seq, __ATOMIC_ACQUIRE) == ctx->cg_seq; };
+    for (unsigned i = 1; !there(); ++i) {
+        if (i & 0xffffu) continue;
+        const cudaError_t e = cudaStreamQuery(ctx->stream);
+        if (e == cudaErrorNotReady) {
+            (void)cudaGetLastError();
+            continue;
+        }
+        KRR_TRY_CUDA(e);
+        if (!there()) return fail(ctx, KRR_E_CUDA, "solve: the scalars of an iteration did not arrive");
+    }
+    return KRR_OK;
+}
+
 int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol, double* alpha,
               krr_solve_info* info) {
     if (!ctx) return KRR_E_INVAL;
@@ -960,6 +979,10 @@ int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol
                     KRR_RET(square_product(ctx, p, nrhs, q, form));
             }
             inf.mvm_count++;
+            ++it;
+            ++since;
+            const bool last = it >= ctx->opts.max_iter;
+            const bool read = it % ctx->opts.check_every == 0 || last;
             {
                 Phase ph(ctx, PH_CGVEC);
                 if (hp) {
@@ -967,26 +990,27 @@ int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol
                     KRR_RET(launch_cg64_update_xr(ctx, x64, rr64, p64, q64, nrhs, part2));
                 } else {
                     KRR_RET(launch_cg_alpha(ctx, p, q, nrhs, part1));
-                    KRR_RET(launch_cg_update_xr(ctx, x, r, p, q, nrhs, part2, 0.0));
+                    KRR_RET(launch_cg_update_xr(ctx, x, r, p, q, nrhs, part2, 0.0, read,
+                                                form == 1 ? tc_err_dev : nullptr));
                 }
             }
-            ++it;
-            ++since;
-            const bool last = it >= ctx->opts.max_iter;
             bool applied = false;
-            if (it % ctx->opts.check_every == 0 || last) {
-                KRR_TRY_CUDA(cudaMemcpyAsync(ctx->cg_host, ctx->cg, sizeof(CGScalars),
-                                             cudaMemcpyDeviceToHost, ctx->stream));
-                if (form == 1)
-                    KRR_TRY_CUDA(cudaMemcpyAsync(tc_err_host, tc_err_dev, sizeof(int),
+            if (read) {
+                if (hp) {
+                    KRR_TRY_CUDA(cudaMemcpyAsync(ctx->cg_host, ctx->cg, sizeof(CGScalars),
                                                  cudaMemcpyDeviceToHost, ctx->stream));
+                    if (form == 1)
+                        KRR_TRY_CUDA(cudaMemcpyAsync(tc_err_host, tc_err_dev, sizeof(int),
+                                                     cudaMemcpyDeviceToHost, ctx->stream));
+                    KRR_TRY_CUDA(cudaEventRecord(ctx->cg_read, ctx->stream));
+                }
                 // The apply of this residual is queued before the host waits for the scalars: the GPU
                 // works while the host decides, and in all but the few iterations that replace the
                 // residual the apply is the one that is needed.
-                KRR_TRY_CUDA(cudaEventRecord(ctx->cg_read, ctx->stream));
                 KRR_RET(apply());
                 applied = true;
-                KRR_TRY_CUDA(cudaEventSynchronize(ctx->cg_read));
+                if (hp) KRR_TRY_CUDA(cudaEventSynchronize(ctx->cg_read));
+                else KRR_RET(wait_mirror(ctx));
                 if (form == 1 && *tc_err_host) {
                     status = KRR_E_TIMEOUT;
                     fail(ctx, status, "tensor-core product: a bounded wait timed out");

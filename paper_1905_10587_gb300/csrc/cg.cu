@@ -542,11 +542,13 @@ __global__ void k_cg_check(CGScalars* cg, const double* __restrict__ part, int n
     __syncthreads();
     if (threadIdx.x == 0) cg->all_done = any ? 0 : 1;
 }
-// x += a p; r -= a q; r.r and, in the last block, the check above
+// x += a p; r -= a q; r.r and, in the last block, the check above.  With `host` (pinned) that block also
+// writes what the host decides on there, and then `seq`: two copies and an event between this kernel
+// and the next cost the queue three more entries an iteration, and the overlap of their launches.
 __global__ void __launch_bounds__(VT)
 k_cg_update_xr(float* __restrict__ x, float* __restrict__ r, const float* __restrict__ p,
                const float* __restrict__ qv, long long n, CGScalars* cg,
-               double* __restrict__ part, double tol2) {
+               double* __restrict__ part, double tol2, CGScalars* host, const int* tc_err, unsigned long long seq) {
     pdl_entry();
     {
         const int q = blockIdx.y;
@@ -571,6 +573,20 @@ k_cg_update_xr(float* __restrict__ x, float* __restrict__ r, const float* __rest
     }
     __syncthreads();
     if (threadIdx.x == 0) cg->all_done = any ? 0 : 1;
+    if (!host) return;
+    if (threadIdx.x < gridDim.y) host->rr[threadIdx.x] = cg->rr[threadIdx.x];
+    if (threadIdx.x == 0) {
+        host->a[0] = cg->a[0];
+        host->b[0] = cg->b[0];
+        host->bad = cg->bad;
+        host->tc_err = tc_err ? *tc_err : 0;
+    }
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence_system();
+        *(volatile unsigned long long*)&host->seq = seq;
+    }
 }
 
 // b_q = rz_new / rz; rz = rz_new (b = 0 for finished columns: p restarts from z)
@@ -662,9 +678,10 @@ int launch_cg_alpha(krr_ctx* ctx, const float* p, const float* q, int nrhs, doub
 }
 
 int launch_cg_update_xr(krr_ctx* ctx, float* x, float* r, const float* p, const float* q, int nrhs,
-                        double* part, double tol2) {
+                        double* part, double tol2, bool mirror, const int* tc_err) {
     const int nb = vec_blocks(ctx, ctx->n);
-    launch_pdl(k_cg_update_xr, dim3(nb, nrhs), VT, 0, ctx->stream, x, r, p, q, ctx->n, ctx->cg, part, tol2);
+    launch_pdl(k_cg_update_xr, dim3(nb, nrhs), VT, 0, ctx->stream, x, r, p, q, ctx->n, ctx->cg, part, tol2,
+               mirror ? ctx->cg_host : nullptr, tc_err, mirror ? ++ctx->cg_seq : 0ull);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }

@@ -66,6 +66,7 @@ struct CGScalars {
     int bad;            // a non-finite or non-positive curvature was met
     int tc_err;         // host mirror only: the tensor-core product's error word
     unsigned ticket[3]; // blocks that have finished, of the passes whose last block forms scalars
+    unsigned long long seq;   // host mirror only: which update of x and r it shows, written last
 };
 
 struct Buf {
@@ -122,7 +123,8 @@ struct krr_ctx {
     unsigned char* FB = nullptr;   // tensor-core features of X (column role)
     krr::CGScalars* cg = nullptr;
     krr::CGScalars* cg_host = nullptr;   // pinned mirror
-    cudaEvent_t cg_read = nullptr;       // the mirror has been written
+    unsigned long long cg_seq = 0;       // updates of x and r that were to write the mirror
+    cudaEvent_t cg_read = nullptr;       // the mirror has been copied (FP64 recurrence)
 
     // ---- phase timers (off unless krr_profile_enable)
     bool prof = false;
