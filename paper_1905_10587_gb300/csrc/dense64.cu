@@ -57,7 +57,8 @@ __device__ __forceinline__ double recip64(double d) {
 // major, lower; identity-padded): A_jj = L L^T.  Elimination keeps A_jj = U^T D U unscaled
 // (v_r = pivot column, d its pivot): a_rc -= v_r (v_c / d), and the same row operations on the
 // identity give the unit inverse; L and its inverse follow from both by the d^(1/2) in parallel.
-// Threads (x, y) of 32 x 8 own column x of rows y, y + 8, ...
+// Threads (x, y) of 32 x 8 own column x of rows y, y + 8, ...  Bound by FP64 issue: the two halves of
+// a row share one instruction (38 us a block with one for each, 32 so).
 constexpr int PF_Y = 8;
 __global__ void __launch_bounds__(NB * PF_Y)
 k_potf2(double* __restrict__ A, int k, int j0, int nb, double tau, int* __restrict__ info,
@@ -85,9 +86,11 @@ k_potf2(double* __restrict__ A, int k, int j0, int nb, double tau, int* __restri
         __syncthreads();
 #pragma unroll
         for (int r = y; r < NB; r += PF_Y) {
-            if (r > m) {
-                if (c > m && c <= r) s[r][c] = fma(-s[r][m], w[c], s[r][c]);
-                else if (c <= m) ei[r][c] = fma(-w[r], ei[m][c], ei[r][c]);
+            if (r > m) {                           // one FMA for both halves of the row
+                const bool right = c > m;
+                double* o = right ? &s[r][c] : &ei[r][c];
+                const double v = fma(right ? -s[r][m] : -w[r], right ? w[c] : ei[m][c], *o);
+                if (c <= r) *o = v;
             }
         }
         __syncthreads();

@@ -315,6 +315,97 @@ k_kgemm(const float* __restrict__ Pr, int nr, const float* __restrict__ Pc, int 
     }
 }
 
+// The same sums, in the same order, by blocks of 32 rows and 64-deep steps, for few points: blocks of
+// 128 rows leave most SMs idle (n = 2000, 110 columns: 16 blocks and 301 us, so 117; n = 4001, 165
+// columns: 64 blocks and 629 us, so 359).
+// A thread has 8 rows x 2 columns, so that a warp's shared reads are two broadcasts and 256 bytes
+// for 16 FMAs; the next step's V is loaded to registers during this one's products.
+constexpr int KS_BM = 32, KS_BK = 64;
+template <int D>
+__global__ void __launch_bounds__(KG_THREADS)
+k_kgemm_few(const float* __restrict__ Pr, int nr, const float* __restrict__ Pc, int nc, const float* __restrict__ V,
+            int ldv, int ncol, float* __restrict__ Out, int ldo) {
+    pdl_entry();
+    constexpr int PS = (D + 1 + 3) / 4 * 4;
+    constexpr int VL = KS_BK * KG_BN / KG_THREADS;      // V values of a step, a thread's
+    constexpr int XL = (KS_BK * PS + KG_THREADS - 1) / KG_THREADS;   // and of the points
+    __shared__ __align__(16) float sXc[KS_BK][PS];
+    __shared__ __align__(16) float sPt[KS_BK][KS_BM];
+    __shared__ __align__(16) float sV[KS_BK][KG_BN];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int rg = (w >> 1) * 8, cg = 2 * (lane + 32 * (w & 1));
+    const long long row0 = (long long)blockIdx.y * KS_BM;
+    const int col0 = blockIdx.x * KG_BN;
+    float xr[D + 1];                                    // the point of row `lane`, whose kernel values it forms
+#pragma unroll
+    for (int c = 0; c <= D; ++c) {
+        xr[c] = (row0 + lane < nr) ? Pr[(row0 + lane) * PS + c] : 0.f;
+        if (c < D) xr[c] *= 2.f;
+    }
+    const int vc = tid % KG_BN, vk = tid / KG_BN;       // this thread's column of V, every second row
+    const bool vin = col0 + vc < ncol;
+    float vr[VL], pr[XL];
+    auto fetch = [&](int j0) {
+#pragma unroll
+        for (int u = 0; u < XL; ++u) {
+            const int e = tid + u * KG_THREADS;
+            pr[u] = e < KS_BK * PS && j0 + e / PS < nc ? Pc[(size_t)j0 * PS + e] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < VL; ++u) {
+            const int j = j0 + vk + u * (KG_THREADS / KG_BN);
+            vr[u] = vin && j < nc ? V[(size_t)j * ldv + col0 + vc] : 0.f;
+        }
+    };
+    fetch(0);
+    float acc[8][2];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) acc[r][0] = acc[r][1] = 0.f;
+    for (int j0 = 0; j0 < nc; j0 += KS_BK) {
+#pragma unroll
+        for (int u = 0; u < XL; ++u)
+            if (tid + u * KG_THREADS < KS_BK * PS) (&sXc[0][0])[tid + u * KG_THREADS] = pr[u];
+#pragma unroll
+        for (int u = 0; u < VL; ++u) sV[vk + u * (KG_THREADS / KG_BN)][vc] = vr[u];
+        __syncthreads();
+        fetch(j0 + KS_BK);
+#pragma unroll 2
+        for (int kk = w; kk < KS_BK; kk += KG_THREADS / 32) {
+            float xc[PS];
+#pragma unroll
+            for (int c = 0; c < PS; c += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(&sXc[kk][c]);
+                xc[c] = v.x, xc[c + 1] = v.y, xc[c + 2] = v.z, xc[c + 3] = v.w;
+            }
+            float t = xr[D] + xc[D];
+#pragma unroll
+            for (int c = 0; c < D; ++c) t = fmaf(xr[c], xc[c], t);
+            sPt[kk][lane] = (j0 + kk < nc) ? ex2f(t) : 0.f;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int kk = 0; kk < KS_BK; ++kk) {
+            const float4 a0 = *reinterpret_cast<const float4*>(&sPt[kk][rg]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&sPt[kk][rg + 4]);
+            const float2 v = *reinterpret_cast<const float2*>(&sV[kk][cg]);
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                acc[r][0] = fmaf(a[r], v.x, acc[r][0]);
+                acc[r][1] = fmaf(a[r], v.y, acc[r][1]);
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const long long i = row0 + rg + r;
+        if (i >= nr) continue;
+        if (col0 + cg < ncol) Out[i * ldo + col0 + cg] = acc[r][0];
+        if (col0 + cg + 1 < ncol) Out[i * ldo + col0 + cg + 1] = acc[r][1];
+    }
+}
+
 typedef void (*kgemm_fn)(const float*, int, const float*, int, const float*, int, int, float*,
                          int);
 
@@ -330,6 +421,17 @@ static kgemm_fn kgemm_pick(int dk) {
     return nullptr;
 }
 
+static kgemm_fn kgemm_few_pick(int dk) {
+    switch (dk) {
+#define KRR_D(v) \
+    case v: return &k_kgemm_few<v>;
+        KRR_D(1) KRR_D(2) KRR_D(3) KRR_D(4) KRR_D(5) KRR_D(6) KRR_D(7) KRR_D(8)
+        KRR_D(9) KRR_D(10) KRR_D(11) KRR_D(12) KRR_D(13) KRR_D(14) KRR_D(15) KRR_D(16)
+#undef KRR_D
+    }
+    return nullptr;
+}
+
 int launch_kgemm(krr_ctx* ctx, const float* Pr, long long nr, const float* Pc, long long nc, int d,
                  const float* V, int ldv, int ncol, float* Out, int ldo) {
     if (nr > 0x7fffffffLL || nc > 0x7fffffffLL)
@@ -338,6 +440,15 @@ int launch_kgemm(krr_ctx* ctx, const float* Pr, long long nr, const float* Pc, l
     if (!fn) return fail(ctx, KRR_E_INVAL, "kgemm: unsupported dimension");
     dim3 grid(ceil_div(ncol, KG_BN), ceil_div(nr, KG_BM));
     if (grid.y > 65535u) return fail(ctx, KRR_E_INVAL, "kgemm: too many row blocks");
+    // fewer blocks of 128 rows than SMs: the kernel of 32-row blocks, where it is compiled (d <= 16;
+    // beyond, its 64-deep tiles of points do not fit)
+    if ((long long)grid.x * grid.y < ctx->num_sms)
+        if (kgemm_fn few = kgemm_few_pick(kernel_dim(d))) {
+            launch_pdl(few, dim3(grid.x, ceil_div(nr, KS_BM)), KG_THREADS, 0, ctx->stream, Pr, (int)nr, Pc, (int)nc,
+                       V, ldv, ncol, Out, ldo);
+            KRR_CHECK_LAUNCH();
+            return KRR_OK;
+        }
     fn<<<grid, KG_THREADS, 0, ctx->stream>>>(Pr, (int)nr, Pc, (int)nc, V, ldv, ncol, Out, ldo);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
@@ -346,14 +457,23 @@ int launch_kgemm(krr_ctx* ctx, const float* Pr, long long nr, const float* Pc, l
 // ------------------------------------------------------------------ Gram  G = beta I + F^T F
 constexpr int GR_THREADS = 256, GR_B = 64, GR_BK = 32, GR_FOLD = 256;
 
+// block (a, b), a >= b, that is number p = a (a + 1) / 2 + b
+__device__ __forceinline__ int2 gram_pair(int p) {
+    int a = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
+    while (a * (a + 1) / 2 > p) --a;
+    while ((a + 1) * (a + 2) / 2 <= p) ++a;
+    return make_int2(a, p - a * (a + 1) / 2);
+}
+
 // One CTA: a 64x64 block (ba, bb), ba >= bb, of F^T F over rows [r0, r1).
 // Products are summed in FP32 over GR_FOLD rows and folded into FP64.
 __global__ void __launch_bounds__(GR_THREADS)
-k_gram(const float* __restrict__ F, long long n, int k, int ldF, const int2* __restrict__ pairs,
-       long long rows_per_split, double* __restrict__ part) {
+k_gram(const float* __restrict__ F, long long n, int k, int ldF, long long rows_per_split,
+       double* __restrict__ part) {
+    pdl_entry();
     __shared__ __align__(16) float sA[GR_BK][GR_B];
     __shared__ __align__(16) float sB[GR_BK][GR_B];
-    const int2 pr = pairs[blockIdx.x];
+    const int2 pr = gram_pair((int)blockIdx.x);
     const int a0 = pr.x * GR_B, b0 = pr.y * GR_B;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const long long r0 = (long long)blockIdx.y * rows_per_split;
@@ -403,50 +523,40 @@ k_gram(const float* __restrict__ F, long long n, int k, int ldF, const int2* __r
             out[(ty * 4 + r) * GR_B + tx * 4 + c] = acc64[r][c] + (double)acc[r][c];
 }
 
-__global__ void k_gram_reduce(const double* __restrict__ part, int splits, int npairs,
-                              const int2* __restrict__ pairs, int k, double beta,
-                              double* __restrict__ G) {
+// G from the splits' sums, a thread an element (a block a pair took 25 us at k = 200)
+constexpr int GRR_T = 256;
+__global__ void __launch_bounds__(GRR_T)
+k_gram_reduce(const double* __restrict__ part, int splits, int npairs, int k, double beta, double* __restrict__ G) {
+    pdl_entry();
     const int p = blockIdx.x;
-    const int2 pr = pairs[p];
-    for (int e = threadIdx.x; e < GR_B * GR_B; e += blockDim.x) {
-        const int r = e / GR_B, c = e - r * GR_B;
-        const int a = pr.x * GR_B + r, b = pr.y * GR_B + c;
-        if (a >= k || b >= k) continue;
-        double s = 0.0;
-        for (int sp = 0; sp < splits; ++sp) s += part[((size_t)sp * npairs + p) * GR_B * GR_B + e];
-        if (a == b) s += beta;
-        G[(size_t)a * k + b] = s;
-        G[(size_t)b * k + a] = s;
-    }
+    const int2 pr = gram_pair(p);
+    const int e = blockIdx.y * GRR_T + threadIdx.x;
+    const int a = pr.x * GR_B + e / GR_B, b = pr.y * GR_B + e % GR_B;
+    if (a >= k || b >= k) return;
+    double s = 0.0;
+#pragma unroll 8
+    for (int sp = 0; sp < splits; ++sp) s += part[((size_t)sp * npairs + p) * GR_B * GR_B + e];
+    if (a == b) s += beta;
+    G[(size_t)a * k + b] = s;
+    G[(size_t)b * k + a] = s;
 }
 
 int launch_gram(krr_ctx* ctx, const float* F, long long n, int k, int ldF, double beta, double* G) {
     const int nb = (k + GR_B - 1) / GR_B;
     const int npairs = nb * (nb + 1) / 2;
-    int2* pairs;
-    KRR_RET(bufT(ctx, "gram_pairs", (size_t)npairs, &pairs));
-    {
-        int2* hp = new int2[npairs];
-        int p = 0;
-        for (int a = 0; a < nb; ++a)
-            for (int b = 0; b <= a; ++b) hp[p++] = make_int2(a, b);
-        cudaError_t e = cudaMemcpyAsync(pairs, hp, sizeof(int2) * npairs, cudaMemcpyHostToDevice,
-                                        ctx->stream);
-        cudaError_t e2 = cudaStreamSynchronize(ctx->stream);
-        delete[] hp;
-        if (e != cudaSuccess || e2 != cudaSuccess)
-            return fail(ctx, KRR_E_CUDA, "gram: pair table upload failed");
-    }
     const int target = 3 * ctx->num_sms * 2;
-    int splits = (int)std::max<long long>(1, std::min<long long>(target / npairs + 1, ceil_div(n, 4 * GR_FOLD)));
+    // splits of at least 128 rows: of 1024, a few thousand rows and few anchors gave 6 to 60 blocks
+    // (with the reduction 142 us at n = 2000, k = 100 and 156 at n = 6000, k = 200; so 21 and 48)
+    int splits = (int)std::max<long long>(1, std::min<long long>(target / npairs + 1, ceil_div(n, 128)));
     const long long rps = ((ceil_div(n, splits) + GR_BK - 1) / GR_BK) * GR_BK;
     splits = (int)ceil_div(n, rps);
     double* part;
     KRR_RET(bufT(ctx, "gram_part", (size_t)splits * npairs * GR_B * GR_B, &part));
     dim3 grid(npairs, splits);
-    k_gram<<<grid, GR_THREADS, 0, ctx->stream>>>(F, n, k, ldF, pairs, rps, part);
+    launch_pdl_if(npairs * splits < target, k_gram, grid, GR_THREADS, 0, ctx->stream, F, n, k, ldF, rps, part);
     KRR_CHECK_LAUNCH();
-    k_gram_reduce<<<npairs, 256, 0, ctx->stream>>>(part, splits, npairs, pairs, k, beta, G);
+    launch_pdl(k_gram_reduce, dim3(npairs, GR_B * GR_B / GRR_T), GRR_T, 0, ctx->stream, part, splits, npairs, k, beta,
+               G);
     KRR_CHECK_LAUNCH();
     return KRR_OK;
 }
