@@ -709,8 +709,8 @@ int launch_kmvm(krr_ctx* ctx, const float* Pr, long long nr, const float* Pc, lo
                                          (double)beta, Q64 + (size_t)(done / 2) * nr, ksc));
         } else if (part) {
             const long long tot = nr * chunk;
-            launch_pdl(k_kmvm_reduce, ceil_div(tot, 256), 256, 0, ctx->stream, part, splits, (int)nr, chunk, Vc,
-                       (int)nc, beta, Qc, (int)nr, ksc);
+            k_kmvm_reduce<<<ceil_div(tot, 256), 256, 0, ctx->stream>>>(part, splits, (int)nr, chunk, Vc, (int)nc,
+                                                                       beta, Qc, (int)nr, ksc);
             KRR_CHECK_LAUNCH();
         }
         done += chunk;
@@ -897,8 +897,8 @@ int kmvm_into_scratch(cudaStream_t stream, int num_sms, const float* Xr, long lo
                                                           (float)beta, 0.f, 0.f, Qc, (int)nr,
                                                           splits > 1 ? part : nullptr);
         if (splits > 1)
-            launch_pdl(k_kmvm_reduce, ceil_div(nr * chunk, 256), 256, 0, stream, part, splits, (int)nr, chunk, Vc,
-                       (int)nc, (float)beta, Qc, (int)nr, 1.0);
+            k_kmvm_reduce<<<ceil_div(nr * chunk, 256), 256, 0, stream>>>(part, splits, (int)nr, chunk, Vc, (int)nc,
+                                                                         (float)beta, Qc, (int)nr, 1.0);
         done += chunk;
     }
     return cudaGetLastError() == cudaSuccess ? KRR_OK : KRR_E_CUDA;
