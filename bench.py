@@ -239,9 +239,9 @@ def run_reference(args):
 # DRAM bytes of one product launch (dram__bytes_read.sum + dram__bytes_write.sum from one
 # ncu capture of the current kernel on this workload): (form, n, d) -> bytes.  Entries are
 # removed whenever the kernel changes and re-taken from a capture of the new one.  The
-# V-folded tensor-core product reads both 64-wide BF16 feature sets (2 x 12.8 MB at n = 10^5)
-# once from DRAM; the column features' re-reads are L2 hits.
-MEASURED_TRAFFIC = {(1, 100000, 8): 25_670_144}
+# symmetric tensor-core product reads both 64-wide BF16 feature sets (2 x 12.8 MB at n = 10^5)
+# once from DRAM; re-reads are L2 hits and most of the partial sums stay there.
+MEASURED_TRAFFIC = {(1, 100000, 8): 26_260_736}
 
 
 # ------------------------------------------------------------------ roofline of the product
@@ -255,6 +255,10 @@ def roofline(p, kms, kcnt, clocks, precision, sms):
     Peak pairs/s = min(FMA-pipe rate / FMA ops per pair, MUFU rate), from
     the SM count x 128 FP32 lanes (resp. 32 ex2 per SM per clock on GB300) x the
     largest SM clock seen.
+
+    One right-hand side on the training points evaluates every unordered pair once for both of
+    its sums.  `achieved` and `peak` count the n^2 pairs (i, j) of the product, as if each took its
+    own ex2; `frac_evaluated` is the fraction of that rate at which the kernel evaluates pairs.
     """
     sm_max = (clocks.get("sm_max_mhz") or 2070.0) * 1e6
     ffma_rate = sms * 128 * sm_max
@@ -264,12 +268,14 @@ def roofline(p, kms, kcnt, clocks, precision, sms):
     peak_pairs = min(ffma_rate / fma_per_pair, mufu_rate)
     avg_s = (kms / max(kcnt, 1)) / 1e3
     achieved = (float(p.n) * p.n / avg_s) if kcnt else None
-    name = ("k_kmvm_tc<1, 16, true> (tcgen05 BF16x3 exponent GEMM with v folded into the exponent, "
-            "ex2 + FADD), (K + beta I) p; the timed phase includes the v partition and the reduction"
-            if precision == 1 else "k_kmvm (tiled FP32 kernel product), (K + beta I) p")
+    name = ("k_kmvm_sym (tcgen05 BF16x3 exponent GEMM, each pair's ex2 used for its row's and its column's "
+            "sum), (K + beta I) p; the timed phase includes the padding of p and the reduction"
+            if precision == 1 else "k_sym_f32 (FP32 kernel product, each pair once), (K + beta I) p")
+    evaluated = 0.5 * achieved * (p.n + 1) / p.n if achieved and nrhs == 1 else achieved
     return {"bound": "alu", "achieved": achieved / 1e9 if achieved else None,
             "peak": peak_pairs / 1e9, "unit": "Gpair/s",
             "frac": (achieved / peak_pairs) if achieved else None,
+            "frac_evaluated": (evaluated / peak_pairs) if achieved else None,
             "traffic": MEASURED_TRAFFIC.get((precision, p.n, p.d)),
             "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
             "kernel": name,
@@ -562,6 +568,8 @@ def cube_extra(api, sms: int, sm_hz: float, reps: int = 3) -> dict:
             ms = e0.elapsed_time(e1) / reps
             rate = float(p.n) ** 2 / (ms / 1e3)
             bound = _alu_bound(sms, sm_hz, _form_fma_ops(prec, p.d, nrhs, bool(tc_pv)))
+            if prec == 1 and nrhs == 1:
+                bound *= 2   # each unordered pair's ex2 serves (i, j) and (j, i)
             key = f"prec{prec}_nrhs{nrhs}" + ("" if tc_pv else "_pv_fma")
             out[key] = {"ms": ms, "pairs_per_s": rate, "frac": rate / bound, "bound_pairs_per_s": bound}
         ctx.close()
