@@ -975,8 +975,13 @@ int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol
                 Phase ph(ctx, PH_KMVM);
                 if (hp)
                     KRR_RET(square_product64(ctx, p64, nrhs, psplit, q64, form));
-                else
-                    KRR_RET(square_product(ctx, p, nrhs, q, form));
+                else {
+                    ctx->have_pq = false;
+                    ctx->want_pq = nrhs == 1;   // a block of columns takes several reductions
+                    const int rc = square_product(ctx, p, nrhs, q, form);
+                    ctx->want_pq = false;
+                    KRR_RET(rc);
+                }
             }
             inf.mvm_count++;
             ++it;
@@ -989,7 +994,7 @@ int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol
                     KRR_RET(launch_cg64_alpha(ctx, p64, q64, nrhs, part1));
                     KRR_RET(launch_cg64_update_xr(ctx, x64, rr64, p64, q64, nrhs, part2));
                 } else {
-                    KRR_RET(launch_cg_alpha(ctx, p, q, nrhs, part1));
+                    if (!ctx->have_pq) KRR_RET(launch_cg_alpha(ctx, p, q, nrhs, part1));
                     KRR_RET(launch_cg_update_xr(ctx, x, r, p, q, nrhs, part2, 0.0, read,
                                                 form == 1 ? tc_err_dev : nullptr));
                 }

@@ -8,7 +8,7 @@
 // with F = K(X, X_S) L1^{-T} stored (n x ldF) and T2 = L2^{-1} held explicitly,
 // so one application is two streaming passes over F and two k x k triangular
 // products in FP64.
-#include "internal.cuh"
+#include "cg_scalar.cuh"
 #include "sym.cuh"
 
 #include <algorithm>
@@ -46,30 +46,6 @@ __device__ __forceinline__ void block_sum_store(double v, double* part, int q) {
         for (int i = 0; i < VT / 32; ++i) s += red[i];
         part[(size_t)q * gridDim.x + blockIdx.x] = s;
     }
-}
-
-// True in every thread of the grid's last block to get here: the blocks' global writes before the
-// call are then visible to it.  *ticket starts at 0 and is 0 again afterwards.
-__device__ __forceinline__ bool last_block(unsigned* ticket) {
-    __shared__ bool last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        last = atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1;
-        if (last) *ticket = 0;
-    }
-    __syncthreads();
-    if (last) __threadfence();
-    return last;
-}
-
-// sum of column q's per-block partials, in every lane (read past L1: another block of the same launch
-// may have written them)
-__device__ __forceinline__ double warp_sum_parts(const double* __restrict__ part, int nblk, int q) {
-    const int lane = threadIdx.x & 31;
-    double s = 0.0;
-    for (int b = lane; b < nblk; b += 32) s += __ldcg(part + (size_t)q * nblk + b);
-    return warp_sum(s);
 }
 
 __global__ void __launch_bounds__(VT)
@@ -479,20 +455,6 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
 // ------------------------------------------------------------------ PCG recurrences
 // The scalar kernels run one warp per right-hand side: the warp sums that column's
 // per-block partials (FP64) and lane 0 applies the recurrence.
-// a_q = rz_q / (p_q . q_q) for active columns; zero otherwise (one warp; s = p_q . q_q).
-__device__ __forceinline__ void cg_alpha(CGScalars* cg, int q, double s) {
-    cg->pq[q] = s;
-    double a = 0.0;
-    if (cg->active[q]) {
-        if (!(s > 0.0) || !isfinite(s) || !isfinite(cg->rz[q])) {
-            cg->bad = 1;
-            cg->active[q] = 0;
-        } else {
-            a = cg->rz[q] / s;
-        }
-    }
-    cg->a[q] = a;
-}
 __global__ void k_cg_alpha(CGScalars* cg, const double* __restrict__ part, int nblk, int nrhs) {
     const int q = threadIdx.x >> 5;
     if (q >= nrhs) return;

@@ -124,6 +124,8 @@ struct krr_ctx {
     krr::CGScalars* cg = nullptr;
     krr::CGScalars* cg_host = nullptr;   // pinned mirror
     unsigned long long cg_seq = 0;       // updates of x and r that were to write the mirror
+    bool want_pq = false;                // a solve's product p -> q: its reduction may form p . q and the step
+    bool have_pq = false;                // and did
     cudaEvent_t cg_read = nullptr;       // the mirror has been copied (FP64 recurrence)
 
     // ---- phase timers (off unless krr_profile_enable)

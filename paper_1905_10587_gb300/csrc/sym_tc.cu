@@ -35,6 +35,7 @@
 // tiles 10% slower.  Fetching v a tile ahead and asking for the next tile's barrier a step ahead
 // gave 5% together, folding row and column sums under the next tile's exponentials 4%.
 #include "internal.cuh"
+#include "cg_scalar.cuh"
 #include "sym.cuh"
 #include "tc_ptx.cuh"
 
@@ -465,14 +466,16 @@ k_kmvm_sym(const unsigned char* __restrict__ FA, const unsigned char* __restrict
 }
 
 // q_i = ksc vscale (sum of point i's column and row slots) + beta v_i (vscale null: 1).  One block per tile: 128 points
-// x 4 interleaved groups of column slots.
+// x 4 interleaved groups of column slots.  With cg also v . q, in whose last block the CG step is formed:
+// a pass of its own over both vectors cost an iteration 5 us (58 of them at n = 6000, k = 200).
 constexpr int SYR_G = 4;
 __global__ void __launch_bounds__(SY_T * SYR_G)
 k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __restrict__ colpart,
              const float* __restrict__ V, float beta, double ksc, const double* __restrict__ vscale,
-             float* __restrict__ Q) {
+             float* __restrict__ Q, CGScalars* cg, double* __restrict__ dpart) {
     pdl_entry();
     __shared__ double red[SYR_G][SY_T];
+    __shared__ double dred[SY_T / 32];
     const int x = threadIdx.x & (SY_T - 1), grp = threadIdx.x / SY_T;
     const int i = blockIdx.x * SY_T + x;
     const int T = i / sg.BN, b = T / sg.RU;
@@ -492,19 +495,42 @@ k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __rest
     }
     red[grp][x] = (double)h + (double)l;
     __syncthreads();
+    double dot = 0.0;
     if (grp == 0 && i < sg.n) {
         double t = red[0][x];
 #pragma unroll
         for (int w = 1; w < SYR_G; ++w) t += red[w][x];
-        Q[i] = (float)(t * (vscale ? ksc * *vscale : ksc) + (beta != 0.f ? (double)beta * V[i] : 0.0));
+        const float v = V[i];
+        const float q = (float)(t * (vscale ? ksc * *vscale : ksc) + (beta != 0.f ? (double)beta * v : 0.0));
+        Q[i] = q;
+        dot = (double)v * (double)q;
     }
+    if (!cg) return;
+    if (grp == 0) {
+        dot = warp_sum(dot);
+        if ((x & 31) == 0) dred[x >> 5] = dot;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < SY_T / 32; ++w) t += dred[w];
+        dpart[blockIdx.x] = t;
+    }
+    if (!last_block(&cg->ticket[1]) || threadIdx.x >= 32) return;
+    const double t = warp_sum_parts(dpart, gridDim.x, 0);
+    if (threadIdx.x == 0) cg_alpha(cg, 0, t);
 }
 
 int launch_sym_reduce(krr_ctx* ctx, const SyGrid& g, const float2* rowpart, const float2* colpart, const float* V,
                       float beta, double ksc, const double* vscale, float* Q) {
-    launch_pdl(k_sym_reduce, g.NU * g.BN / SY_T, SY_T * SYR_G, 0, ctx->stream, g, rowpart, colpart, V, beta, ksc,
-               vscale, Q);
+    const int blocks = g.NU * g.BN / SY_T;
+    double* dpart = nullptr;
+    if (ctx->want_pq) KRR_RET(bufT(ctx, "sym_dot", (size_t)blocks, &dpart));
+    launch_pdl(k_sym_reduce, blocks, SY_T * SYR_G, 0, ctx->stream, g, rowpart, colpart, V, beta, ksc, vscale, Q,
+               dpart ? ctx->cg : nullptr, dpart);
     KRR_CHECK_LAUNCH();
+    ctx->have_pq = ctx->want_pq;
     return KRR_OK;
 }
 

@@ -47,3 +47,19 @@ def test_chained_applications(n, k, r):
         out.append(V.cpu())
     assert torch.equal(out[0], out[1])
     assert torch.isfinite(out[0]).all()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n,r", [(1, 1), (127, 1), (129, 1), (1025, 1), (300, 3)])
+def test_solve_with_the_step_from_the_reduction(n, r, precision):
+    """One column takes p . q and its step from the product's reduction, a block of columns does not.
+    Bar: the tolerance, with 1e-3 of it for the float-float residual that the solve stops on."""
+    from paper_1905_10587_gb300.api import KRR
+    X, Y = _data(n, 4, r)
+    ctx = KRR(precision=precision)
+    ctx.build(X, 2.0, 1e-2, max(1, n // 10), seed=5)
+    alpha, _ = ctx.solve(Y, tol=1e-6)
+    Xd, a = X.double(), alpha.double().reshape(n, r)
+    A = torch.exp(-torch.cdist(Xd, Xd, compute_mode="donot_use_mm_for_euclid_dist") ** 2 / 8.0)
+    res = Y.double() - A @ a - 1e-2 * a
+    assert (res.norm(dim=0) / Y.double().norm(dim=0)).max().item() <= 1.001e-6
