@@ -442,9 +442,8 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
         KRR_RET(launch_tri_gemv(ctx, ctx->T2, k, u, nq, true, u1));
         KRR_RET(launch_tri_gemv(ctx, ctx->T2t, k, u1, nq, false, v));
         const size_t smem = sizeof(float4) * nq * (ldF / 4);
-        if (smem > 48 * 1024) {
-            KRR_RET(allow_max_dynamic_smem(ctx, (const void*)gn));
-        }
+        // always: the 48 KB that need no leave are for the dynamic and the kernel's static memory together
+        KRR_RET(allow_max_dynamic_smem(ctx, (const void*)gn));
         launch_pdl_if(nb < 4 * ctx->num_sms, gn, nb, VT, smem, ctx->stream, ctx->F, n, k, ldF, v, Rq, n, inv_beta, Zq,
                    rz_part ? rz_part + (size_t)q0 * nb : nullptr, rz_part && with_beta ? ctx->cg : nullptr, q0);
         KRR_CHECK_LAUNCH();
