@@ -404,6 +404,18 @@ typedef void (*gemv_n_fn)(const float*, long long, int, int, const double*, cons
                           float, float*, double*, CGScalars*, int);
 constexpr int AP_NQ = 8;   // most right-hand sides per pass over F
 
+// Right-hand sides per pass over F: r - F v holds v of all of them in shared memory (4 ldF bytes each,
+// beside up to 1 KB of sums), so that more than about 7200 anchors leave room for fewer than eight.
+// As many as fit: a pass reads F once whatever its columns, and one block an SM with eight is still
+// ahead of two passes (n = 30000, eight columns, against passes of four with more blocks an SM:
+// k = 3800 0.98 against 1.42 ms, 5000 1.34 against 1.87, 6500 1.87 against 2.65).
+static int apply_columns(krr_ctx* ctx, int ldF, int* nq) {
+    int optin = 0;
+    KRR_TRY_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+    *nq = std::max(1, std::min(AP_NQ, (optin - 2048) / (4 * ldF)));
+    return KRR_OK;
+}
+
 // Z = M^{-1} R for nrhs columns.  When rz_part is non-null it receives per-block partial
 // sums of R.Z laid out [q][blk] with apply_blocks(ctx) blocks per column; with_beta also forms the
 // recurrence's b and rz_new from them.
@@ -415,7 +427,9 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
     const int CW = std::min(VT, ldF / 4);          // threads across a row of F
     float2* upart;
     double *u, *u1, *v;
-    const int mq = std::min(AP_NQ, nrhs);
+    int mq;
+    KRR_RET(apply_columns(ctx, ldF, &mq));
+    mq = std::min(mq, nrhs);
     KRR_RET(bufT(ctx, "ap_upart2", (size_t)nt * mq * ldF, &upart));
     KRR_RET(bufT(ctx, "ap_u", (size_t)mq * k, &u));
     KRR_RET(bufT(ctx, "ap_u1", (size_t)mq * k, &u1));
@@ -429,8 +443,8 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
     static const gemv_n_fn gns[AP_NQ] = {&k_gemv_n_apply<1>, &k_gemv_n_apply<2>, &k_gemv_n_apply<3>,
                                          &k_gemv_n_apply<4>, &k_gemv_n_apply<5>, &k_gemv_n_apply<6>,
                                          &k_gemv_n_apply<7>, &k_gemv_n_apply<8>};
-    for (int q0 = 0; q0 < nrhs; q0 += AP_NQ) {
-        const int nq = std::min(AP_NQ, nrhs - q0);
+    for (int q0 = 0; q0 < nrhs; q0 += mq) {
+        const int nq = std::min(mq, nrhs - q0);
         const gemv_t_fn gt = gts[2 * CW > VT][nq - 1];   // room for one row group only
         const gemv_n_fn gn = gns[nq - 1];
         const float* Rq = R + (size_t)q0 * n;

@@ -49,3 +49,9 @@ def test_apply_just_below_48_kilobytes():
     assert len(got) == len(NEAR_48K)
     for k, r, e in got:
         assert float(e) <= 1.0, (k, r, e)
+
+
+# from about 7200 anchors eight columns do not fit the shared memory of a block; 7 + 2 columns at k = 8000
+@pytest.mark.parametrize("k,nrhs", [(7100, 8), (8000, 8), (8000, 9)])
+def test_apply_with_many_anchors(k, nrhs):
+    assert backward(k, nrhs) <= 1.0
