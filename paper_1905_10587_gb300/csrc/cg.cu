@@ -213,8 +213,28 @@ k_gemv_t(const float* __restrict__ F, long long n, int ldF, const float* __restr
 // threads: each group sums every 32nd partial (8 consecutive columns = one 64-byte
 // segment per load), and the groups combine through shared memory.  k / 8 CTAs keep
 // enough loads in flight for the 4 x SMs partials of the F^T r pass.
-__device__ __forceinline__ double part_value(double v) { return v; }
-__device__ __forceinline__ double part_value(float2 v) { return (double)v.x + (double)v.y; }
+// Pairs are added as pairs and converted once: a conversion of both halves of each cost four FP64
+// instructions a partial sum (70 cycles each for a warp here).  A whole apply at n = 30000, k = 1000
+// with FP64 partial sums, with each pair converted, and so: two columns 93, 114 and 87 us, three 129,
+// 140 and 112, eight (two passes of four with FP64 ones) 388, 230 and 208.  The pair's 2^-44 a term is
+// far below the FP32 entries of F: against 64 bits the apply is as far off as with FP64 sums.
+template <class T>
+struct PartSum;
+template <>
+struct PartSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double v) { s += v; }
+    __device__ __forceinline__ double get() const { return s; }
+};
+template <>
+struct PartSum<float2> {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float2 v) {
+        ff_add(h, l, v.x);
+        l = __fadd_rn(l, v.y);
+    }
+    __device__ __forceinline__ double get() const { return (double)h + (double)l; }
+};
 template <class T>
 __global__ void __launch_bounds__(256)
 k_gemv_t_reduce(const T* __restrict__ upart, int nblk, int nq, int k, int ldF,
@@ -224,10 +244,10 @@ k_gemv_t_reduce(const T* __restrict__ upart, int nblk, int nq, int k, int ldF,
     const int c = threadIdx.x & 7, g = threadIdx.x >> 3;
     const int a = blockIdx.x * 8 + c;
     const int q = blockIdx.y;
-    double s = 0.0;
+    PartSum<T> sum;
     if (a < k)
-        for (int b = g; b < nblk; b += 32) s += part_value(upart[((size_t)b * nq + q) * ldF + a]);
-    red[g][c] = s;
+        for (int b = g; b < nblk; b += 32) sum.add(upart[((size_t)b * nq + q) * ldF + a]);
+    red[g][c] = sum.get();
     __syncthreads();
     if (threadIdx.x < 8 && a < k) {
         double t = 0.0;
@@ -408,7 +428,7 @@ constexpr int AP_NQ = 8;   // most right-hand sides per pass over F
 // beside up to 1 KB of sums), so that more than about 7200 anchors leave room for fewer than eight.
 // As many as fit: a pass reads F once whatever its columns, and one block an SM with eight is still
 // ahead of two passes (n = 30000, eight columns, against passes of four with more blocks an SM:
-// k = 3800 0.98 against 1.42 ms, 5000 1.34 against 1.87, 6500 1.87 against 2.65).
+// k = 3800 0.89 against 1.42 ms, 5000 1.21 against 1.87, 6500 1.70 against 2.65).
 static int apply_columns(krr_ctx* ctx, int ldF, int* nq) {
     int optin = 0;
     KRR_TRY_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));

@@ -55,3 +55,29 @@ def test_apply_just_below_48_kilobytes():
 @pytest.mark.parametrize("k,nrhs", [(7100, 8), (8000, 8), (8000, 9)])
 def test_apply_with_many_anchors(k, nrhs):
     assert backward(k, nrhs) <= 1.0
+
+
+# partial sums of F^T r from every number of blocks up to the most there are (four an SM), with few and
+# many columns a pass; the backward error against the Nystrom K~ of the same anchors in FP64
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 8])
+@pytest.mark.parametrize("n,k", [(33, 20), (1025, 90), (20011, 600), (60013, 300)])
+def test_apply_partial_sums(n, k, nrhs, sigma=1.0, beta=1e-2):
+    from paper_1905_10587_gb300.api import KRR
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + nrhs)
+    X = torch.randn((n, 8), generator=g, device="cuda")
+    V = torch.randn((n, nrhs), generator=g, device="cuda")
+    ctx = KRR(pivot_tol=0.0)
+    ctx.build(X, sigma, beta, k, anchors=torch.arange(k, device="cuda", dtype=torch.int32))
+    z = ctx.apply_precond(V).double()
+    ctx.close()
+    Xd = X.double()
+    C = torch.exp(-torch.cdist(Xd, Xd[:k], compute_mode="donot_use_mm_for_euclid_dist") ** 2 / (2 * sigma**2))
+    L = torch.linalg.cholesky(C[:k])
+    F = torch.linalg.solve_triangular(L, C.t(), upper=False)
+    v = torch.ones(n, dtype=torch.float64, device="cuda")
+    for _ in range(30):                       # a lower bound of ||K~||
+        v = F.t() @ (F @ (v / v.norm()))
+    r = (F.t() @ (F @ z) + beta * z - V.double()).norm(dim=0)
+    eta = (2 * (k + 5) + k + 2) * 2.0**-24
+    assert (r / (eta * (v.norm() + beta) * z.norm(dim=0))).max().item() <= 1.0
