@@ -66,8 +66,16 @@ __device__ __forceinline__ void sy_fma(unsigned long long& d, unsigned long long
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 
+// The points of an FP32 product as its kernel has them (packed, or raw coordinates with nsc != 0), for
+// the sums that leave the range of its float pairs; P null where v was scaled so that none does.
+struct SyPoints {
+    const float* P = nullptr;
+    int d = 0, ps = 0;
+    float nsc = 0.f;
+};
+
 // Q = ksc vscale (row and column partial sums) + beta V (vscale: device, null for 1)
 int launch_sym_reduce(krr_ctx* ctx, const SyGrid& g, const float2* rowpart, const float2* colpart, const float* V,
-                      float beta, double ksc, const double* vscale, float* Q);
+                      float beta, double ksc, const double* vscale, float* Q, SyPoints pts = SyPoints());
 
 }  // namespace krr

@@ -281,7 +281,12 @@ int launch_kmvm_sym_f32(krr_ctx* ctx, const float* P, long long n, int d, float 
     KRR_RET(bufT(ctx, "sy_col", (size_t)g.col_base(g.NU), &colpart));
     launch_pdl(fn, g.G, threads, 0, ctx->stream, P, g, V, raw_nsc, rowpart, colpart);
     KRR_CHECK_LAUNCH();
-    return launch_sym_reduce(ctx, g, rowpart, colpart, V, beta, 1.0, nullptr, Q);
+    SyPoints pts;
+    pts.P = P;
+    pts.d = kernel_dim(d);
+    pts.ps = packed_stride(d);
+    pts.nsc = raw_nsc;
+    return launch_sym_reduce(ctx, g, rowpart, colpart, V, beta, 1.0, nullptr, Q, pts);
 }
 
 }  // namespace krr

@@ -468,11 +468,28 @@ k_kmvm_sym(const unsigned char* __restrict__ FA, const unsigned char* __restrict
 // q_i = ksc vscale (sum of point i's column and row slots) + beta v_i (vscale null: 1).  One block per tile: 128 points
 // x 4 interleaved groups of column slots.  With cg also v . q, in whose last block the CG step is formed:
 // a pass of its own over both vectors cost an iteration 5 us (58 of them at n = 6000, k = 200).
+// A float pair that overflowed, or met an infinity, holds Inf - Inf in its low half, and a sum of both
+// signs may overflow on the way to a finite value.  Points with such a slot are summed again from the
+// points themselves in FP64, where the kernel has them (pts.P: FP32 products; the tensor-core product
+// scales v, so that only an infinity in v gets there, and takes the high half): exact-form
+// semantics for the price of one flag a block otherwise.
 constexpr int SYR_G = 4;
+__device__ __noinline__ double sy_exact_sum(SyPoints pts, const float* V, int n, int i, int j0) {
+    double s = 0.0;
+    const float* x = pts.P + (size_t)i * pts.ps;
+    for (int j = j0; j < n; j += SYR_G) {
+        const float* y = pts.P + (size_t)j * pts.ps;
+        float t = pts.nsc != 0.f ? 0.f : x[pts.d] + y[pts.d];
+        for (int c = 0; c < pts.d; ++c)
+            t = pts.nsc != 0.f ? fmaf(x[c] - y[c], x[c] - y[c], t) : fmaf(2.f * x[c], y[c], t);
+        s = fma((double)ex2f(pts.nsc != 0.f ? pts.nsc * t : t), (double)V[j], s);
+    }
+    return s;
+}
 __global__ void __launch_bounds__(SY_T * SYR_G)
 k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __restrict__ colpart,
              const float* __restrict__ V, float beta, double ksc, const double* __restrict__ vscale,
-             float* __restrict__ Q, CGScalars* cg, double* __restrict__ dpart) {
+             float* __restrict__ Q, CGScalars* cg, double* __restrict__ dpart, SyPoints pts) {
     pdl_entry();
     __shared__ double red[SYR_G][SY_T];
     __shared__ double dred[SY_T / 32];
@@ -493,8 +510,17 @@ k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __rest
         ff_add(h, l, w.x);
         l += w.y;
     }
-    red[grp][x] = (double)h + (double)l;
-    __syncthreads();
+    const bool over = !(fabsf(h) <= 3.402823466e38f);
+    red[grp][x] = over ? (double)h : (double)h + (double)l;
+    if (__syncthreads_or(over && pts.P)) {         // rare
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < SYR_G; ++w) t += red[w][x];
+        const bool redo = i < sg.n && !isfinite(t);
+        __syncthreads();
+        if (redo) red[grp][x] = sy_exact_sum(pts, V, sg.n, i, grp);
+        __syncthreads();
+    }
     double dot = 0.0;
     if (grp == 0 && i < sg.n) {
         double t = red[0][x];
@@ -523,12 +549,12 @@ k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __rest
 }
 
 int launch_sym_reduce(krr_ctx* ctx, const SyGrid& g, const float2* rowpart, const float2* colpart, const float* V,
-                      float beta, double ksc, const double* vscale, float* Q) {
+                      float beta, double ksc, const double* vscale, float* Q, SyPoints pts) {
     const int blocks = g.NU * g.BN / SY_T;
     double* dpart = nullptr;
     if (ctx->want_pq) KRR_RET(bufT(ctx, "sym_dot", (size_t)blocks, &dpart));
     launch_pdl(k_sym_reduce, blocks, SY_T * SYR_G, 0, ctx->stream, g, rowpart, colpart, V, beta, ksc, vscale, Q,
-               dpart ? ctx->cg : nullptr, dpart);
+               dpart ? ctx->cg : nullptr, dpart, pts);
     KRR_CHECK_LAUNCH();
     ctx->have_pq = ctx->want_pq;
     return KRR_OK;
