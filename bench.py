@@ -340,7 +340,8 @@ def run_gpu(args):
         tctx = api.KRR(precision=args.precision)
         tctx.build(X, p.sigma, p.beta, p.k, seed=1)
         width = 64 if args.precision == 1 else p.X.shape[1]
-        key = f"form={args.precision} w={width} r=1 lg={int(np.floor(np.log2(p.n)))}"
+        form = 3 if args.precision == 1 else args.precision   # 3: one point set on the tensor cores
+        key = f"form={form} w={width} r=1 lg={int(np.floor(np.log2(p.n)))}"
         got = api.tune_get(key)
         if got is None:
             tctx.autotune(nrhs=1, reps=3)

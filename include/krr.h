@@ -428,8 +428,9 @@ int krr_batch_solve_grouped(const krr_problem* probs, int nprob, int nrhs, doubl
  * opts.autotune = 1.  Keys read "form=F w=W r=R lg=L": product form F (0 FP32
  * expansion, 1 tensor cores, 2 exact differences), feature width W (tensor-core K,
  * else the kernel dimension), R right-hand sides per launch, L = floor(log2 n).
- * (The tensor-core product with R = 1 splits one sequence of work evenly; its count is the
- * height of its row blocks, in 256 points, or 128 with 128-wide features; up to 4.)
+ * Form 3 is the tensor-core product of one point set with R = 1, which splits one sequence of
+ * work evenly: its count is the height of its row blocks, in 256 points, or 128 with 128-wide
+ * features; up to 4.  (The FP32 products of one point set and one column have no entry.)
  * Entries hold the split count, the P.V form (1 = on tensor cores) and the time.
  * The table is process-wide and guarded by a lock.
  *
@@ -438,6 +439,8 @@ int krr_batch_solve_grouped(const krr_problem* probs, int nprob, int nrhs, doubl
  * choice and split counts 1 .. 64, and with 64-wide tensor-core features for both P.V
  * forms; each candidate is run once to warm up, then reps times between CUDA events.
  * Stores the fastest under its key and writes it to the host outputs (each may be NULL).
+ * With nrhs = 1 that is the form for any two point sets; on the tensor cores form 3 is
+ * timed and stored besides.
  * KRR_E_STATE before a build, KRR_E_INVAL for a bad nrhs or reps outside 1 .. 100.
  * krr_tune_save / krr_tune_load write and read the table as JSON (load adds entries;
  * KRR_E_INVAL on a missing file or an entry that does not parse, with nothing added).

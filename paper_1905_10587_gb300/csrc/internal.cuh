@@ -110,6 +110,7 @@ struct krr_ctx {
     int force_splits = 0;      // > 0: this column-split count
     int force_pv = -1;         // >= 0: P.V form of the tensor-core product (1 tensor cores)
     int last_splits = 0;       // split count of the last product launch
+    bool general = false;      // krr_autotune: products of one point set take the form for two
     // device arrays (views into bufs)
     float* P = nullptr;        // n x ps packed points of X
     float* Praw = nullptr;     // n x ps raw coordinates of X (difference form), on demand
@@ -312,13 +313,15 @@ bool sym_f32_fits(long long n, int d);
 int launch_kmvm_sym_f32(krr_ctx* ctx, const float* P, long long n, int d, float beta, const float* V, float* Q,
                         float raw_nsc);
 
-// tune.cu: tuned work splits.  Key of a product configuration; the table entry for it
+// tune.cu: tuned work splits.  Key of a product configuration (form 0 to 2: column splits of the
+// product of any two point sets; kFormSym: row-block height of sym_tc.cu); the table entry for it
 // (only with opts.autotune and outside tuning); the split count to use (forced, tuned or
 // the cost model's `analytic`, clamped to [1, ntiles]; also recorded in ctx->last_splits).
 struct TuneEntry {
     int splits, pv;
     double ms;
 };
+constexpr int kFormSym = 3;
 std::string tune_key(int form, int width, int nrhs, long long n);
 bool tune_lookup(const krr_ctx* ctx, const std::string& key, TuneEntry* out);
 int tuned_splits(krr_ctx* ctx, const std::string& key, int analytic, int ntiles);

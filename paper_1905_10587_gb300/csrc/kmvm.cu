@@ -668,11 +668,11 @@ int launch_kmvm(krr_ctx* ctx, const float* Pr, long long nr, const float* Pc, lo
         const int chunk = comp ? (left >= 4 ? 4 : 2)
                                : left >= 16 ? 16 : left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
         // one right-hand side, one point set: each pair once (see sym_f32.cu)
-        if (chunk == 1 && !hp && Pr == Pc && nr == nc && sym_f32_fits(nr, d)) {
+        if (chunk == 1 && !hp && Pr == Pc && nr == nc && !ctx->general && sym_f32_fits(nr, d)) {
             const int rc = launch_kmvm_sym_f32(ctx, Pr, nr, d, beta, V + (size_t)done * nc, Q + (size_t)done * nr,
                                                raw_nsc);
-            ctx->last_splits = 1;
             if (rc == KRR_OK) {
+                ctx->last_splits = 1;
                 done += chunk;
                 continue;
             }

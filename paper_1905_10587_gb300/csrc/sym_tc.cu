@@ -620,7 +620,8 @@ int launch_kmvm_sym(krr_ctx* ctx, const unsigned char* FA, const unsigned char* 
             best = RU;
         }
     }
-    const int RU = std::max(rumin, tuned_splits(ctx, tune_key(1, Kp, 1, n), best, rumax));
+    const int RU = std::max(rumin, tuned_splits(ctx, tune_key(kFormSym, Kp, 1, n), best, rumax));
+    ctx->last_splits = RU;
     const SyGrid g = make(RU);
     const int np = g.NU * BN;
     const int nbmax = (int)ceil_div(np, SY_PAD);

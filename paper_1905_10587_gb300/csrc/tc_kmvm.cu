@@ -1496,6 +1496,18 @@ int launch_kmvm_tc(krr_ctx* ctx, const unsigned char* FA, long long nr, const un
         const int left = nrhs - done;
         const int chunk = left >= 16 ? 16 : left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
         const std::string key = tune_key(1, Kp, chunk, nr);
+        // one column on one point set: each pair once (sym_tc.cu).  The table's P.V form for this key is
+        // that of the product of two sets.
+        const bool sym = chunk == 1 && !hp && same && !ctx->general && ctx->opts.tc_pv != 2 && sym_tc_fits(nr);
+        if (sym) {
+            const int rc = launch_kmvm_sym(ctx, FA, FB, nr, d, beta, V + (size_t)done * nc, Q + (size_t)done * nr, err);
+            if (rc == KRR_OK) {
+                done += chunk;
+                continue;
+            }
+            if (rc != KRR_E_NOMEM) return rc;   // no room for its partial sums: the forms below
+            ctx->err.clear();
+        }
         bool use_pv = !hp && Kp == 64 && (ctx->opts.tc_pv == 2 || (ctx->opts.tc_pv == 1 && chunk >= 8));
         TuneEntry te;
         if (!hp && Kp == 64) {
@@ -1507,15 +1519,6 @@ int launch_kmvm_tc(krr_ctx* ctx, const unsigned char* FA, long long nr, const un
                                      Q + (size_t)done * nr, err));
             done += chunk;
             continue;
-        }
-        if (chunk == 1 && !hp && same && sym_tc_fits(nr)) {
-            const int rc = launch_kmvm_sym(ctx, FA, FB, nr, d, beta, V + (size_t)done * nc, Q + (size_t)done * nr, err);
-            if (rc == KRR_OK) {
-                done += chunk;
-                continue;
-            }
-            if (rc != KRR_E_NOMEM) return rc;   // no room for its partial sums: the form below
-            ctx->err.clear();
         }
         // 16 epilogue warps (32 would need 34 warps with the producer and the MMA issuer,
         // above the 32 warps a CTA may have)

@@ -5,6 +5,8 @@
 // overhead.  krr_autotune times the candidates for the built problem of a context instead
 // and keeps the fastest in a process-wide table keyed by
 //     (product form, feature width, right-hand sides per launch, floor(log2 n)),
+// (the tensor-core product of one point set and one column, which is cut evenly whatever its count,
+// is a form of its own, with the height of its row blocks in the place of the count)
 // which later products of the same key use when opts.autotune = 1.  The table can be
 // written to and read from a JSON file, so tuned choices carry over between processes.
 #include "internal.cuh"
@@ -89,37 +91,46 @@ extern "C" int krr_autotune(krr_ctx* ctx, int nrhs, int reps, int* splits_out, i
     KRR_RET(bufT(ctx, "tune_q", (size_t)n * nrhs, &Q));
     k_tune_fill<<<(unsigned)ceil_div(n * nrhs, 256), 256, 0, ctx->stream>>>(V, n * nrhs);
     KRR_CHECK_LAUNCH();
-    // candidates: the cost model's own choice (0) and a spread of split counts; with
-    // tensor-core features of width 64, both P.V forms
-    const int cand[] = {0, 1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
-    std::vector<int> pvs = {-1};
-    if (form == 1 && width == 64) pvs = {0, 1};
     cudaEvent_t e0, e1;
     KRR_TRY_CUDA(cudaEventCreate(&e0));
     KRR_TRY_CUDA(cudaEventCreate(&e1));
     ctx->tuning = true;
-    TuneEntry best{0, 0, HUGE_VAL};
     int rc = KRR_OK;
-    for (int pv : pvs) {
-        for (int c : cand) {
-            ctx->force_splits = c;
-            ctx->force_pv = pv;
-            rc = square_product(ctx, V, nrhs, Q, form);   // warm-up (and allocations)
-            if (rc != KRR_OK) break;
-            const int used = ctx->last_splits;
-            if (c > 0 && used != c) continue;               // beyond the tile count
-            cudaEventRecord(e0, ctx->stream);
-            for (int r = 0; r < reps && rc == KRR_OK; ++r) rc = square_product(ctx, V, nrhs, Q, form);
-            cudaEventRecord(e1, ctx->stream);
-            if (cudaEventSynchronize(e1) != cudaSuccess) rc = KRR_E_CUDA;
-            if (rc != KRR_OK) break;
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            const double t = ms / reps;
-            if (t < best.ms) best = TuneEntry{used, pv < 0 ? 0 : pv, t};
-        }
-        if (rc != KRR_OK) break;
-    }
+    // the fastest of the counts (0: the cost model's own choice) and P.V forms
+    auto fastest = [&](const std::vector<int>& counts, const std::vector<int>& pvs) {
+        TuneEntry best{0, 0, HUGE_VAL};
+        for (int pv : pvs)
+            for (int c : counts) {
+                if (rc != KRR_OK) break;
+                ctx->force_splits = c;
+                ctx->force_pv = pv;
+                rc = square_product(ctx, V, nrhs, Q, form);   // warm-up (and allocations)
+                if (rc != KRR_OK) break;
+                const int used = ctx->last_splits;
+                if (c > 0 && used != c) continue;               // beyond the tile count
+                cudaEventRecord(e0, ctx->stream);
+                for (int r = 0; r < reps && rc == KRR_OK; ++r) rc = square_product(ctx, V, nrhs, Q, form);
+                cudaEventRecord(e1, ctx->stream);
+                if (cudaEventSynchronize(e1) != cudaSuccess) rc = KRR_E_CUDA;
+                if (rc != KRR_OK) break;
+                float ms = 0.f;
+                cudaEventElapsedTime(&ms, e0, e1);
+                const double t = ms / reps;
+                if (t < best.ms) best = TuneEntry{used, pv < 0 ? 0 : pv, t};
+            }
+        return best;
+    };
+    // column splits of the product of two point sets, which a product of one set with more than one
+    // column takes too; with tensor-core features of width 64, both P.V forms
+    ctx->general = true;
+    const TuneEntry best = fastest({0, 1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64},
+                                   form == 1 && width == 64 ? std::vector<int>{0, 1} : std::vector<int>{-1});
+    ctx->general = false;
+    // one column on one point set has a form and a key of its own on the tensor cores (the FP32 one
+    // has nothing to choose)
+    TuneEntry height{0, 0, HUGE_VAL};
+    if (rc == KRR_OK && form == 1 && nrhs == 1 && ctx->opts.tc_pv != 2 && sym_tc_fits(n))
+        height = fastest({0, 1, 2, 3, 4}, {-1});
     ctx->tuning = false;
     ctx->force_splits = 0;
     ctx->force_pv = -1;
@@ -127,6 +138,7 @@ extern "C" int krr_autotune(krr_ctx* ctx, int nrhs, int reps, int* splits_out, i
     cudaEventDestroy(e1);
     if (rc != KRR_OK) return rc;
     tune_store(tune_key(form, width, nrhs, n), best);
+    if (height.splits > 0) tune_store(tune_key(kFormSym, width, 1, n), height);
     if (splits_out) *splits_out = best.splits;
     if (pv_out) *pv_out = best.pv;
     if (ms_out) *ms_out = best.ms;
