@@ -24,7 +24,9 @@
  *     column r of an n x nrhs block starts at ptr + r * n.
  *   - A context owns its device workspace (allocated with cudaMalloc, grown on
  *     demand, released by krr_destroy) and issues all work on the stream given
- *     to krr_create.  A context is not thread-safe.
+ *     to krr_create.  A context is not thread-safe.  The workspace grows with n k
+ *     and n nrhs; the products that evaluate each pair of a point set once hold
+ *     at most 256 MB of partial sums.
  *   - Return value: KRR_OK or a KRR_E_* code.  Nothing aborts or throws; the
  *     message of the last failure is available from krr_last_error().
  *   - Preconditions are checked on the host before any launch: n >= 1,

@@ -306,6 +306,7 @@ int square_product(krr_ctx* ctx, const float* V, int nrhs, float* Q, int form) {
 
 static int build_common(krr_ctx* ctx, const float* X, long long n, int d, double sigma,
                         double beta) {
+    ctx->sym_nomem = 0;
     ctx->built = false;
     ctx->X = X;
     ctx->n = n;
@@ -461,6 +462,7 @@ long long krr_launch_count(const krr_ctx* ctx) { return ctx ? ctx->launches : 0;
 int krr_kmvm(krr_ctx* ctx, const float* Xr, long long nr, const float* Xc, long long nc, int d,
              double sigma, double beta, const float* V, int nrhs, float* Q) {
     if (!ctx) return KRR_E_INVAL;
+    ctx->sym_nomem = 0;
     KRR_RET(check_points(ctx, Xr, nr, d));
     KRR_RET(check_points(ctx, Xc, nc, d));
     KRR_RET(check_sigma_beta(ctx, sigma, beta, false));
@@ -773,6 +775,7 @@ static int wait_mirror(krr_ctx* ctx) {
 int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol, double* alpha,
               krr_solve_info* info) {
     if (!ctx) return KRR_E_INVAL;
+    ctx->sym_nomem = 0;
     if (!ctx->built) return fail(ctx, KRR_E_STATE, "krr_solve before krr_build_precond");
     if (X != ctx->X) return fail(ctx, KRR_E_INVAL, "X differs from the built point set");
     if (!Y || !alpha) return fail(ctx, KRR_E_INVAL, "null Y or alpha");

@@ -110,6 +110,8 @@ struct krr_ctx {
     int force_splits = 0;      // > 0: this column-split count
     int force_pv = -1;         // >= 0: P.V form of the tensor-core product (1 tensor cores)
     int last_splits = 0;       // split count of the last product launch
+    size_t sym_nomem = 0;      // > 0: partial sums of this size did not fit the device (sym.cuh); a new
+                               // call of krr_kmvm, krr_solve or a build tries again
     bool general = false;      // krr_autotune: products of one point set take the form for two
     // device arrays (views into bufs)
     float* P = nullptr;        // n x ps packed points of X

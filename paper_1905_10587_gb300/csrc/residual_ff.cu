@@ -22,6 +22,7 @@
 #include "sym.cuh"
 
 #include <algorithm>
+#include <type_traits>
 #include <cmath>
 
 namespace krr {
@@ -229,9 +230,9 @@ template <int R>
 constexpr int sff_bn() { return R == 1 ? 64 : 128; }
 constexpr int SFF_T = 256, SFF_NW = SFF_T / 32;
 
-template <int D, int MODE, int R>
+template <int D, int MODE, int R, class Grid>
 __global__ void __launch_bounds__(SFF_T, 2)
-k_sym_ff(const float* __restrict__ X, SyGrid sg, const float2* __restrict__ N2, float sh, float sl,
+k_sym_ff(const float* __restrict__ X, Grid sg, const float2* __restrict__ N2, float sh, float sl,
          const float2* __restrict__ Aff, const FfTab tab, double* __restrict__ rowpart,
          double* __restrict__ colpart) {
     constexpr int BN = sff_bn<R>(), RB = 8 * SFF_NW * R;
@@ -319,47 +320,62 @@ k_sym_ff(const float* __restrict__ X, SyGrid sg, const float2* __restrict__ N2, 
             }
 #pragma unroll
             for (int r = 0; r < R; ++r) acc[r] += (double)Sh[r] + (double)Sl[r];
-            at = T / sg.RU > I ? sg.col_base(T) + (long long)I * BN : -1;
+            at = T / sg.RU > I ? sg.col_base(T) + (long long)sg.slot(I) * BN : -1;
         }
 #pragma unroll
         for (int r = 0; r < R; ++r) {              // over the four column groups
             double x = acc[r];
             x += __shfl_xor_sync(0xffffffffu, x, 8);
             x += __shfl_xor_sync(0xffffffffu, x, 16);
-            if (lc == 0) rowpart[(long long)(run + I) * RB + w * 8 * R + 8 * r + lr] = x;
+            if (lc == 0) rowpart[(long long)(run + sg.slot(I)) * RB + w * 8 * R + 8 * r + lr] = x;
         }
     }
     __syncthreads();
     store_column((cc & 1) ^ 1);
 }
 
-// Point i's slots in a fixed order; out = scale S (Y null) or Y - beta A - S.
+// Point i's slots in a fixed order; out = scale S (Y null) or Y - beta A - S.  With panels acc holds the
+// sums of those before, and out is written after the last.
+template <class Grid>
 __global__ void __launch_bounds__(256)
-k_sym_ff_reduce(SyGrid sg, const double* __restrict__ rowpart, const double* __restrict__ colpart, double scale,
-                const float* __restrict__ Y, const double* __restrict__ A, double beta, double* __restrict__ out) {
+k_sym_ff_reduce(Grid sg, const double* __restrict__ rowpart, const double* __restrict__ colpart, double scale,
+                const float* __restrict__ Y, const double* __restrict__ A, double beta, double* __restrict__ out,
+                double* __restrict__ acc) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= sg.n) return;
     const int T = i / sg.BN, b = T / sg.RU;
     const double* cp = colpart + sg.col_base(T) + i % sg.BN;
     double s = 0.0;
 #pragma unroll 4
-    for (int I = 0; I < b; ++I) s += cp[(long long)I * sg.BN];
-    const int s0 = sg.run_of(sg.first(b)), s1 = sg.run_of(sg.first(b + 1) - 1);
-    for (int r = s0; r <= s1; ++r) s += rowpart[(long long)(r + b) * sg.rows() + i % sg.rows()];
+    for (int I = 0; I < sg.slots(b); ++I) s += cp[(long long)I * sg.BN];
+    if (sg.has(b)) {
+        const int s0 = sg.run_of(sg.first(b)), s1 = sg.run_of(sg.first(b + 1) - 1);
+        for (int r = s0; r <= s1; ++r) s += rowpart[(long long)(r + sg.slot(b)) * sg.rows() + i % sg.rows()];
+    }
+    if (!sg.first_panel()) s += acc[i];
+    if (!sg.last_panel()) {
+        acc[i] = s;
+        return;
+    }
     out[i] = Y ? (double)Y[i] - beta * A[i] - s : scale * s;
 }
 
-typedef void (*sff_fn)(const float*, SyGrid, const float2*, float, float, const float2*, FfTab, double*,
-                       double*);
-template <int D>
-static sff_fn sff_pick1(int mode, int R) {
-    if (mode == 0) return R == 4 ? &k_sym_ff<D, 0, 4> : R == 2 ? &k_sym_ff<D, 0, 2> : &k_sym_ff<D, 0, 1>;
-    return R == 4 ? &k_sym_ff<D, 1, 4> : R == 2 ? &k_sym_ff<D, 1, 2> : &k_sym_ff<D, 1, 1>;
+template <class Grid>
+using sff_fn = void (*)(const float*, Grid, const float2*, float, float, const float2*, FfTab, double*, double*);
+template <int D, class Grid>
+static sff_fn<Grid> sff_pick1(int mode, int R) {
+    if (R == 4) return mode == 0 ? &k_sym_ff<D, 0, 4, Grid> : &k_sym_ff<D, 1, 4, Grid>;
+    if constexpr (std::is_same<Grid, SyGrid>::value) {   // panels are for large sets, with four rows
+        if (mode == 0) return R == 2 ? &k_sym_ff<D, 0, 2, Grid> : &k_sym_ff<D, 0, 1, Grid>;
+        return R == 2 ? &k_sym_ff<D, 1, 2, Grid> : &k_sym_ff<D, 1, 1, Grid>;
+    }
+    return nullptr;
 }
-static sff_fn sff_pick(int d, int mode, int R) {
+template <class Grid>
+static sff_fn<Grid> sff_pick(int d, int mode, int R) {
     switch (d) {
 #define KRR_D(v) \
-    case v: return sff_pick1<v>(mode, R);
+    case v: return sff_pick1<v, Grid>(mode, R);
         KRR_D(1) KRR_D(2) KRR_D(3) KRR_D(4) KRR_D(5) KRR_D(6) KRR_D(7) KRR_D(8)
         KRR_D(9) KRR_D(10) KRR_D(11) KRR_D(12) KRR_D(13) KRR_D(14) KRR_D(15) KRR_D(16)
 #undef KRR_D
@@ -462,12 +478,12 @@ int kernel_occupancy(const void* fn, int threads);   // kmvm.cu
 static int sym_ff(krr_ctx* ctx, const float* X, long long n, int d, double sigma, const double* A, int mode,
                   double out_scale, const float* Y, double beta, double* out, bool* ran) {
     *ran = false;
-    if (n > (1LL << 19)) return KRR_OK;            // partial sums take n^2 / 64 bytes
+    if (n > (1LL << 19)) return KRR_OK;
     SyGrid g{}, best{};
-    sff_fn fn = nullptr;
+    int bestR = 0;
     double best_cost = 0.0;
     for (int R = 4; R >= 1; R /= 2) {
-        const sff_fn f = sff_pick(d, mode, R);
+        const sff_fn<SyGrid> f = sff_pick<SyGrid>(d, mode, R);
         if (!f) return fail(ctx, KRR_E_INVAL, "float-float product: unsupported shape");
         const int RB = 8 * SFF_NW * R;
         g.n = (int)n;
@@ -480,35 +496,44 @@ static int sym_ff(krr_ctx* ctx, const float* X, long long n, int d, double sigma
         // the longest run sets the time: units x (pairs, and a column's lane sum per R rows)
         const double cost = (double)((g.W + g.G - 1) / g.G) * RB * g.BN * (1.0 + 0.2 / R) *
                             ((g.G + ctx->num_sms - 1) / ctx->num_sms);
-        if (!fn || cost < best_cost) {
+        if (8 * g.col_base(g.NU) > kSymBytes && R < 4) break;   // panels have four rows
+        if (!bestR || cost < best_cost) {
             best_cost = cost;
             best = g;
-            fn = f;
+            bestR = R;
         }
     }
     g = best;
     float2 *N2, *Aff;
-    double *rowpart, *colpart;
-    const int rc1 = bufT(ctx, "sff_row", (size_t)(g.G + g.nblk) * g.rows(), &rowpart);
-    const int rc2 = bufT(ctx, "sff_col", (size_t)g.col_base(g.NU), &colpart);
-    if (rc1 == KRR_E_NOMEM || rc2 == KRR_E_NOMEM) {
+    double* acc = nullptr;
+    if (8 * g.col_base(g.NU) > kSymBytes) KRR_RET(bufT(ctx, "sym_acc", (size_t)n, &acc));
+    KRR_RET(bufT(ctx, "ff_nr", (size_t)n, &N2));
+    KRR_RET(bufT(ctx, "ff_alpha", (size_t)n, &Aff));
+    const double s = 1.4426950408889634 / (2.0 * sigma * sigma);
+    const float sh = (float)s, sl = (float)(s - (double)sh);
+    bool split = false;
+    const int rc = sym_product(ctx, g, [&](const auto& p, void* row, void* col) -> int {
+        using Grid = std::decay_t<decltype(p)>;
+        double *rowpart = (double*)row, *colpart = (double*)col;
+        if (!split) {
+            k_ff_norms<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(X, n, d, N2);
+            KRR_CHECK_LAUNCH();
+            k_split64<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(A, n, Aff);
+            KRR_CHECK_LAUNCH();
+            split = true;
+        }
+        sff_pick<Grid>(d, mode, bestR)<<<p.G, SFF_T, 0, ctx->stream>>>(X, p, N2, sh, sl, Aff, ff_table(), rowpart, colpart);
+        KRR_CHECK_LAUNCH();
+        k_sym_ff_reduce<Grid><<<ceil_div(n, 256), 256, 0, ctx->stream>>>(p, rowpart, colpart, out_scale, Y, A, beta, out,
+                                                                         acc);
+        KRR_CHECK_LAUNCH();
+        return KRR_OK;
+    });
+    if (rc == KRR_E_NOMEM) {                       // of sym_buffers, before any launch
         ctx->err.clear();
         return KRR_OK;
     }
-    KRR_RET(rc1);
-    KRR_RET(rc2);
-    KRR_RET(bufT(ctx, "ff_nr", (size_t)n, &N2));
-    KRR_RET(bufT(ctx, "ff_alpha", (size_t)n, &Aff));
-    k_ff_norms<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(X, n, d, N2);
-    KRR_CHECK_LAUNCH();
-    k_split64<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(A, n, Aff);
-    KRR_CHECK_LAUNCH();
-    const double s = 1.4426950408889634 / (2.0 * sigma * sigma);
-    const float sh = (float)s, sl = (float)(s - (double)sh);
-    fn<<<g.G, SFF_T, 0, ctx->stream>>>(X, g, N2, sh, sl, Aff, ff_table(), rowpart, colpart);
-    KRR_CHECK_LAUNCH();
-    k_sym_ff_reduce<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(g, rowpart, colpart, out_scale, Y, A, beta, out);
-    KRR_CHECK_LAUNCH();
+    KRR_RET(rc);
     *ran = true;
     return KRR_OK;
 }

@@ -36,7 +36,57 @@ struct SyGrid {
         const long long b = T / RU, r = T % RU;
         return BN * (RU * (b * (b - 1) / 2) + r * b);
     }
+    // the slot of row block I, and the slots of a column unit of block b
+    __host__ __device__ int slot(int I) const { return I; }
+    __host__ __device__ int slots(int b) const { return b; }
+    __host__ __device__ bool first_panel() const { return true; }
+    __host__ __device__ bool last_panel() const { return true; }
+    __host__ __device__ bool has(int) const { return true; }
     static __host__ __device__ int min(int a, int b) { return a < b ? a : b; }
+};
+
+// Most bytes of column sums that a context holds for the products of one point set.  Without a limit
+// they grew as 4 n^2 / rows() (4 GB at n = 10^6 with 1024-row blocks, 16 GB with 256).  256 MB are the
+// sums of 2.6 10^5 points on the tensor cores with 64-wide features, of 1.8 10^5 with 128-wide ones and
+// of 1.3 10^5 in FP32; larger sets take the row blocks in panels, a launch and a reduction each.
+// d = 8, in panels and with all sums (0.6 GB) held: FP32, n = 2 10^5 9.97 and 9.70 ms; tensor cores,
+// n = 4 10^5 14.2 and 14.4 ms.
+constexpr long long kSymBytes = 256LL << 20;
+
+// The row blocks I0 .. I1 - 1 of a grid, whose W pairs from number u0 on are cut into G runs.  A type of
+// its own, for which the kernels are compiled again: the plain one's addresses stay as short as they are.
+struct SyPanel : SyGrid {
+    int I0, I1;
+    long long u0;
+    __host__ __device__ long long run_begin(int s) const { return u0 + W * s / G; }
+    __host__ __device__ int run_of(long long u) const { return (int)(((u - u0 + 1) * G - 1) / W); }
+    __host__ __device__ int slot(int I) const { return I - I0; }
+    __host__ __device__ int slots(int b) const { return b <= I0 ? 0 : min(b, I1) - I0; }
+    __host__ __device__ long long col_base(int T) const {
+        const long long m = slots(T / RU), units = T - (I0 + m) * RU;   // units with m slots before T
+        return m == 0 ? 0 : BN * (RU * (m * (m - 1) / 2) + units * m);
+    }
+    __host__ __device__ bool first_panel() const { return I0 == 0; }
+    __host__ __device__ bool last_panel() const { return I1 == nblk; }
+    __host__ __device__ bool has(int b) const { return b >= I0 && b < I1; }
+    long long col_entries() const {
+        const long long m = I1 - I0, beyond = NU - (long long)I1 * RU;
+        return BN * (RU * (m * (m - 1) / 2) + (beyond > 0 ? beyond : 0) * m);
+    }
+    // The panel from row block I on: as many blocks as `entries` column sums hold, one at least, in up to
+    // maxruns runs.
+    SyPanel(const SyGrid& g, int I, long long entries, int maxruns) : SyGrid(g), I0(I) {
+        int lo = I0 + 1, hi = nblk;                // the entries grow with the blocks
+        while (lo < hi) {
+            I1 = lo + (hi - lo + 1) / 2;
+            if (col_entries() <= entries) lo = I1;
+            else hi = I1 - 1;
+        }
+        I1 = lo;
+        u0 = first(I0);
+        W = first(I1) - u0;
+        G = (int)(W < maxruns ? W : maxruns);
+    }
 };
 
 // Sums each a[m] over the lanes that differ in bit ST and the lower bits halved in turn, down to
@@ -74,8 +124,29 @@ struct SyPoints {
     float nsc = 0.f;
 };
 
-// Q = ksc vscale (row and column partial sums) + beta V (vscale: device, null for 1)
-int launch_sym_reduce(krr_ctx* ctx, const SyGrid& g, const float2* rowpart, const float2* colpart, const float* V,
-                      float beta, double ksc, const double* vscale, float* Q, SyPoints pts = SyPoints());
+// The two buffers of partial sums of a product of up to G runs, shared by all forms (8 bytes an entry).
+// KRR_E_NOMEM where they do not fit the device, without another try while krr_ctx::sym_nomem says so.
+int sym_buffers(krr_ctx* ctx, const SyGrid& g, void** row, void** col);
+
+// Q = ksc vscale (row and column partial sums) + beta V (vscale: device, null for 1), or with a panel that
+// is not the last the running sums.  Defined in sym_tc.cu for SyGrid and SyPanel.
+template <class Grid>
+int launch_sym_reduce(krr_ctx* ctx, const Grid& g, const float2* rowpart, const float2* colpart, const float* V,
+                      float beta, double ksc, const double* vscale, float* Q, SyPoints pts);
+
+// One product in all of its launches: f(grid, rowpart, colpart) for the grid as it is or for each panel,
+// on the buffers that all of them share.
+template <class F>
+inline int sym_product(krr_ctx* ctx, const SyGrid& g, F&& f) {
+    void *row, *col;
+    KRR_RET(sym_buffers(ctx, g, &row, &col));
+    if (8 * g.col_base(g.NU) <= kSymBytes) return f(g, row, col);
+    for (int I = 0; I < g.nblk;) {
+        const SyPanel p(g, I, kSymBytes / 8, g.G);
+        KRR_RET(f(p, row, col));
+        I = p.I1;
+    }
+    return KRR_OK;
+}
 
 }  // namespace krr

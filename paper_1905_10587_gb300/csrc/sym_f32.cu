@@ -26,6 +26,7 @@
 #include "sym.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace krr {
 
@@ -54,9 +55,9 @@ __device__ __forceinline__ unsigned long long sf_mul(unsigned long long a, unsig
 }
 
 // RAW as for k_kmvm2: P holds the caller's coordinates and the exponent is nsc ||x_i - x_j||^2.
-template <int D, int R, bool RAW>
+template <int D, int R, bool RAW, class Grid>
 __global__ void __launch_bounds__(SF_ROWS / R * 4)
-k_sym_f32(const float* __restrict__ P, SyGrid sg, const float* __restrict__ V, float nsc,
+k_sym_f32(const float* __restrict__ P, Grid sg, const float* __restrict__ V, float nsc,
           float2* __restrict__ rowpart, float2* __restrict__ colpart) {
     pdl_entry();
     constexpr int NT = SF_ROWS / R * 4;            // threads
@@ -212,7 +213,7 @@ k_sym_f32(const float* __restrict__ P, SyGrid sg, const float* __restrict__ V, f
             }
             if (more) stage(b ^ 1);
             // inside the diagonal block both triangles were evaluated: row sums only
-            at = T / sg.RU > I ? sg.col_base(T) + (long long)I * SY_T : -1;
+            at = T / sg.RU > I ? sg.col_base(T) + (long long)sg.slot(I) * SY_T : -1;
         }
         // the piece's row sums, over the four column groups
 #pragma unroll
@@ -224,7 +225,7 @@ k_sym_f32(const float* __restrict__ P, SyGrid sg, const float* __restrict__ V, f
                 ff_add(h, l, oh);
                 l += ol;
             }
-            if (lc == 0) rowpart[(long long)(run + I) * SF_ROWS + w * 8 * R + lr + 8 * r] = make_float2(h, l);
+            if (lc == 0) rowpart[(long long)(run + sg.slot(I)) * SF_ROWS + w * 8 * R + lr + 8 * r] = make_float2(h, l);
         }
         ++I;
     }
@@ -232,7 +233,8 @@ k_sym_f32(const float* __restrict__ P, SyGrid sg, const float* __restrict__ V, f
     store_column((cc & 1) ^ 1);
 }
 
-typedef void (*sf_fn)(const float*, SyGrid, const float*, float, float2*, float2*);
+template <class Grid>
+using sf_fn = void (*)(const float*, Grid, const float*, float, float2*, float2*);
 
 // Eight rows per thread halve the shared loads and lane sums per entry, at up to 254 registers (two
 // blocks a SM).  Measured at n = 30011 (us, whole call): expansion d = 12 326 against 352 with four
@@ -240,15 +242,16 @@ typedef void (*sf_fn)(const float*, SyGrid, const float*, float, float2*, float2
 // d = 16 747 against 726, and at n = 8000 80 against 72, so they take four above d = 10.
 template <int D, bool RAW>
 constexpr int sf_rows() { return RAW && D > 10 ? 4 : 8; }
-template <int D>
-static sf_fn sf_pick1(bool raw, int* R) {
+template <int D, class Grid>
+static sf_fn<Grid> sf_pick1(bool raw, int* R) {
     *R = raw ? sf_rows<D, true>() : sf_rows<D, false>();
-    return raw ? &k_sym_f32<D, sf_rows<D, true>(), true> : &k_sym_f32<D, sf_rows<D, false>(), false>;
+    return raw ? &k_sym_f32<D, sf_rows<D, true>(), true, Grid> : &k_sym_f32<D, sf_rows<D, false>(), false, Grid>;
 }
-static sf_fn sf_pick(int dk, bool raw, int* R) {
+template <class Grid>
+static sf_fn<Grid> sf_pick(int dk, bool raw, int* R) {
     switch (dk) {
 #define KRR_D(v) \
-    case v: return sf_pick1<v>(raw, R);
+    case v: return sf_pick1<v, Grid>(raw, R);
         KRR_D(1) KRR_D(2) KRR_D(3) KRR_D(4) KRR_D(5) KRR_D(6) KRR_D(7) KRR_D(8)
         KRR_D(9) KRR_D(10) KRR_D(11) KRR_D(12) KRR_D(13) KRR_D(14) KRR_D(15) KRR_D(16)
 #undef KRR_D
@@ -258,14 +261,14 @@ static sf_fn sf_pick(int dk, bool raw, int* R) {
 
 int kernel_occupancy(const void* fn, int threads);   // kmvm.cu
 
-// Whether the symmetric form takes a square product (its partial sums take n^2 / 64 bytes).
+// Whether the symmetric form takes a square product.
 bool sym_f32_fits(long long n, int d) { return kernel_dim(d) <= 16 && n <= (1LL << 19); }
 
 // Q = (K + beta I) V for packed points P (raw_nsc = 0) or raw coordinates (raw_nsc = -s).
 int launch_kmvm_sym_f32(krr_ctx* ctx, const float* P, long long n, int d, float beta, const float* V, float* Q,
                         float raw_nsc) {
     int R = 8;
-    const sf_fn fn = sf_pick(kernel_dim(d), raw_nsc != 0.f, &R);
+    const sf_fn<SyGrid> fn = sf_pick<SyGrid>(kernel_dim(d), raw_nsc != 0.f, &R);
     if (!fn) return fail(ctx, KRR_E_INVAL, "symmetric product: unsupported dimension");
     const int threads = SF_ROWS / R * 4;
     SyGrid g{};
@@ -276,17 +279,19 @@ int launch_kmvm_sym_f32(krr_ctx* ctx, const float* P, long long n, int d, float 
     g.nblk = g.NU / g.RU;
     g.W = g.first(g.nblk);
     g.G = (int)std::min<long long>(g.W, (long long)ctx->num_sms * kernel_occupancy((const void*)fn, threads));
-    float2 *rowpart, *colpart;
-    KRR_RET(bufT(ctx, "sy_row", (size_t)(g.G + g.nblk) * g.rows(), &rowpart));
-    KRR_RET(bufT(ctx, "sy_col", (size_t)g.col_base(g.NU), &colpart));
-    launch_pdl(fn, g.G, threads, 0, ctx->stream, P, g, V, raw_nsc, rowpart, colpart);
-    KRR_CHECK_LAUNCH();
     SyPoints pts;
     pts.P = P;
     pts.d = kernel_dim(d);
     pts.ps = packed_stride(d);
     pts.nsc = raw_nsc;
-    return launch_sym_reduce(ctx, g, rowpart, colpart, V, beta, 1.0, nullptr, Q, pts);
+    return sym_product(ctx, g, [&](const auto& p, void* row, void* col) -> int {
+        using Grid = std::decay_t<decltype(p)>;
+        float2 *rowpart = (float2*)row, *colpart = (float2*)col;
+        launch_pdl(sf_pick<Grid>(kernel_dim(d), raw_nsc != 0.f, &R), p.G, threads, 0, ctx->stream, P, p, V, raw_nsc, rowpart,
+                   colpart);
+        KRR_CHECK_LAUNCH();
+        return launch_sym_reduce(ctx, p, rowpart, colpart, V, beta, 1.0, nullptr, Q, pts);
+    });
 }
 
 }  // namespace krr

@@ -88,9 +88,9 @@ __global__ void __launch_bounds__(SY_PAD) k_sym_pad(const float* __restrict__ V,
 //   c_full[g][i]             column half g's four column sums in buffer i
 // Every wait is bounded.  A warp whose wait ran out sets the abort and error words and goes on
 // without waiting, so that the block barriers below still match.
-template <int NK, int BN>
+template <int NK, int BN, class Grid>
 __global__ void __launch_bounds__(SY_THREADS, 1)
-k_kmvm_sym(const unsigned char* __restrict__ FA, const unsigned char* __restrict__ FB, int Kp, SyGrid sg,
+k_kmvm_sym(const unsigned char* __restrict__ FA, const unsigned char* __restrict__ FB, int Kp, Grid sg,
            const float* __restrict__ Vp, float2* __restrict__ rowpart, float2* __restrict__ colpart,
            const float* __restrict__ bmax, int nbmax, double* __restrict__ vscale, int* __restrict__ err,
            long long wlimit, int stall_copies) {
@@ -337,7 +337,7 @@ k_kmvm_sym(const unsigned char* __restrict__ FA, const unsigned char* __restrict
             const int ct0 = I * sg.RU + (u - uI), ncol = ue - u;
             const float* vrow = Vp + (size_t)I * R + quarter * 32 + lr;
             float2* srow = sRow + half * R + lrow;
-            float2* cout = colpart + sg.col_base(ct0) + (long long)I * BN;   // this unit's slot
+            float2* cout = colpart + sg.col_base(ct0) + (long long)sg.slot(I) * BN;   // this unit's slot
             int cb = ct0 / sg.RU, cr = ct0 % sg.RU;
             float vn[4];
 #pragma unroll
@@ -423,7 +423,7 @@ k_kmvm_sym(const unsigned char* __restrict__ FA, const unsigned char* __restrict
                 if (lane == 0) mbar_arrive(&sh->b_empty[s]);
                 column_done();
                 slot_at = cb > I ? cout : nullptr;   // right of the diagonal block
-                cout += (long long)cb * BN;          // a unit of block cb has cb slots
+                cout += (long long)sg.slots(cb) * BN;
                 if (++cr == sg.RU) {
                     cr = 0;
                     ++cb;
@@ -442,7 +442,7 @@ k_kmvm_sym(const unsigned char* __restrict__ FA, const unsigned char* __restrict
                 const float2 y = sRow[R + row];
                 ff_add(x.x, x.y, y.x);
                 x.y += y.y;
-                rowpart[(long long)(run + I) * R + row] = x;
+                rowpart[(long long)(run + sg.slot(I)) * R + row] = x;
             }
             sy_bar(1, 32 * SY_EW);
             // nothing is pending: the next fold writes a zero where the next piece starts anew
@@ -486,10 +486,12 @@ __device__ __noinline__ double sy_exact_sum(SyPoints pts, const float* V, int n,
     }
     return s;
 }
+// With panels acc holds the sums of those before (the first writes it), and Q is written after the last.
+template <class Grid>
 __global__ void __launch_bounds__(SY_T * SYR_G)
-k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __restrict__ colpart,
+k_sym_reduce(Grid sg, const float2* __restrict__ rowpart, const float2* __restrict__ colpart,
              const float* __restrict__ V, float beta, double ksc, const double* __restrict__ vscale,
-             float* __restrict__ Q, CGScalars* cg, double* __restrict__ dpart, SyPoints pts) {
+             float* __restrict__ Q, CGScalars* cg, double* __restrict__ dpart, SyPoints pts, double* __restrict__ acc) {
     pdl_entry();
     __shared__ double red[SYR_G][SY_T];
     __shared__ double dred[SY_T / 32];
@@ -497,22 +499,31 @@ k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __rest
     const int i = blockIdx.x * SY_T + x;
     const int T = i / sg.BN, b = T / sg.RU;
     const float2* cp = colpart + sg.col_base(T) + i % sg.BN;
+    const int nslot = sg.slots(b);
     float h = 0.f, l = 0.f;
 #pragma unroll 4
-    for (int I = grp; I < b; I += SYR_G) {
+    for (int I = grp; I < nslot; I += SYR_G) {
         const float2 w = cp[(long long)I * sg.BN];
         ff_add(h, l, w.x);
         l += w.y;
     }
-    const int s0 = sg.run_of(sg.first(b)), s1 = sg.run_of(sg.first(b + 1) - 1);
-    for (int s = s0 + grp; s <= s1; s += SYR_G) {
-        const float2 w = rowpart[(long long)(s + b) * sg.rows() + i % sg.rows()];
-        ff_add(h, l, w.x);
-        l += w.y;
+    if (sg.has(b)) {
+        const int s0 = sg.run_of(sg.first(b)), s1 = sg.run_of(sg.first(b + 1) - 1);
+        for (int s = s0 + grp; s <= s1; s += SYR_G) {
+            const float2 w = rowpart[(long long)(s + sg.slot(b)) * sg.rows() + i % sg.rows()];
+            ff_add(h, l, w.x);
+            l += w.y;
+        }
     }
-    const bool over = !(fabsf(h) <= 3.402823466e38f);
-    red[grp][x] = over ? (double)h : (double)h + (double)l;
-    if (__syncthreads_or(over && pts.P)) {         // rare
+    bool over = !(fabsf(h) <= 3.402823466e38f);
+    double v64 = over ? (double)h : (double)h + (double)l;
+    if (!sg.first_panel() && grp == 0 && i < sg.n) {
+        v64 += acc[i];
+        over = over || !isfinite(v64);             // a panel before was
+    }
+    red[grp][x] = v64;
+    const bool last = sg.last_panel();
+    if (__syncthreads_or(over && last && pts.P)) {   // rare
         double t = 0.0;
 #pragma unroll
         for (int w = 0; w < SYR_G; ++w) t += red[w][x];
@@ -526,12 +537,16 @@ k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __rest
         double t = red[0][x];
 #pragma unroll
         for (int w = 1; w < SYR_G; ++w) t += red[w][x];
+        if (!last) {
+            acc[i] = t;
+            return;
+        }
         const float v = V[i];
         const float q = (float)(t * (vscale ? ksc * *vscale : ksc) + (beta != 0.f ? (double)beta * v : 0.0));
         Q[i] = q;
         dot = (double)v * (double)q;
     }
-    if (!cg) return;
+    if (!cg || !last) return;
     if (grp == 0) {
         dot = warp_sum(dot);
         if ((x & 31) == 0) dred[x >> 5] = dot;
@@ -548,16 +563,34 @@ k_sym_reduce(SyGrid sg, const float2* __restrict__ rowpart, const float2* __rest
     if (threadIdx.x == 0) cg_alpha(cg, 0, t);
 }
 
-int launch_sym_reduce(krr_ctx* ctx, const SyGrid& g, const float2* rowpart, const float2* colpart, const float* V,
+template <class Grid>
+int launch_sym_reduce(krr_ctx* ctx, const Grid& g, const float2* rowpart, const float2* colpart, const float* V,
                       float beta, double ksc, const double* vscale, float* Q, SyPoints pts) {
     const int blocks = g.NU * g.BN / SY_T;
-    double* dpart = nullptr;
-    if (ctx->want_pq) KRR_RET(bufT(ctx, "sym_dot", (size_t)blocks, &dpart));
-    launch_pdl(k_sym_reduce, blocks, SY_T * SYR_G, 0, ctx->stream, g, rowpart, colpart, V, beta, ksc, vscale, Q,
-               dpart ? ctx->cg : nullptr, dpart, pts);
+    const bool pq = ctx->want_pq && g.last_panel();
+    double *dpart = nullptr, *acc = nullptr;
+    if (pq) KRR_RET(bufT(ctx, "sym_dot", (size_t)blocks, &dpart));
+    if (!g.first_panel() || !g.last_panel()) KRR_RET(bufT(ctx, "sym_acc", (size_t)g.n, &acc));
+    launch_pdl(&k_sym_reduce<Grid>, blocks, SY_T * SYR_G, 0, ctx->stream, g, rowpart, colpart, V, beta, ksc, vscale, Q,
+               dpart ? ctx->cg : nullptr, dpart, pts, acc);
     KRR_CHECK_LAUNCH();
-    ctx->have_pq = ctx->want_pq;
+    ctx->have_pq = pq;
     return KRR_OK;
+}
+template int launch_sym_reduce(krr_ctx*, const SyGrid&, const float2*, const float2*, const float*, float, double,
+                               const double*, float*, SyPoints);
+template int launch_sym_reduce(krr_ctx*, const SyPanel&, const float2*, const float2*, const float*, float, double,
+                               const double*, float*, SyPoints);
+
+int sym_buffers(krr_ctx* ctx, const SyGrid& g, void** row, void** col) {
+    const size_t nr = 8 * (size_t)(g.G + g.nblk) * g.rows();
+    const size_t nc = 8 * (size_t)std::min<long long>(g.col_base(g.NU), kSymBytes / 8);
+    if (ctx->sym_nomem && nr + nc >= ctx->sym_nomem)
+        return fail(ctx, KRR_E_NOMEM, "symmetric product: no room for its partial sums");
+    int rc = buf(ctx, "sy_row", nr, row);
+    if (rc == KRR_OK) rc = buf(ctx, "sy_col", nc, col);
+    if (rc == KRR_E_NOMEM) ctx->sym_nomem = nr + nc;
+    return rc;
 }
 
 static size_t sym_smem(int Kp, int BN, int RU) {
@@ -569,23 +602,25 @@ static size_t sym_smem(int Kp, int BN, int RU) {
 
 double ex2_bias_scale(const krr_ctx* ctx);
 
-typedef void (*sym_fn)(const unsigned char*, const unsigned char*, int, SyGrid, const float*, float2*, float2*,
-                       const float*, int, double*, int*, long long, int);
-static sym_fn sym_pick(int nk) {
+template <class Grid>
+using sym_fn = void (*)(const unsigned char*, const unsigned char*, int, Grid, const float*, float2*, float2*,
+                        const float*, int, double*, int*, long long, int);
+template <class Grid>
+static sym_fn<Grid> sym_pick(int nk) {
     switch (nk) {
-        case 1: return &k_kmvm_sym<1, 256>;
-        case 2: return &k_kmvm_sym<2, 256>;
-        case 3: return &k_kmvm_sym<3, 256>;
-        case 4: return &k_kmvm_sym<4, 256>;
-        case 5: return &k_kmvm_sym<5, 128>;
-        case 6: return &k_kmvm_sym<6, 128>;
-        case 7: return &k_kmvm_sym<7, 128>;
+        case 1: return &k_kmvm_sym<1, 256, Grid>;
+        case 2: return &k_kmvm_sym<2, 256, Grid>;
+        case 3: return &k_kmvm_sym<3, 256, Grid>;
+        case 4: return &k_kmvm_sym<4, 256, Grid>;
+        case 5: return &k_kmvm_sym<5, 128, Grid>;
+        case 6: return &k_kmvm_sym<6, 128, Grid>;
+        case 7: return &k_kmvm_sym<7, 128, Grid>;
     }
     return nullptr;
 }
 
 // Whether the symmetric form takes a square product of n points: it is the faster one at every
-// size; its partial sums take 4 n^2 / 1024 bytes (16 GB at the limit, past which k_kmvm_tc runs).
+// size measured; past the limit k_kmvm_tc runs.
 bool sym_tc_fits(long long n) { return n <= (1LL << 21); }
 
 int launch_kmvm_sym(krr_ctx* ctx, const unsigned char* FA, const unsigned char* FB, long long n, int d,
@@ -595,8 +630,7 @@ int launch_kmvm_sym(krr_ctx* ctx, const unsigned char* FA, const unsigned char* 
     // 128-wide features (d >= 10) leave room for two 128-column stages only
     const int BN = Kp == 64 ? 256 : 128;
     const int rumin = 2 * SY_T / BN, rumax = (Kp == 64 ? SY_RTMAX : 4) * SY_T / BN;   // by shared memory
-    const sym_fn fn = sym_pick(nk);
-    if (!fn) return fail(ctx, KRR_E_INVAL, "symmetric product: unsupported dimension");
+    if (!sym_pick<SyGrid>(nk)) return fail(ctx, KRR_E_INVAL, "symmetric product: unsupported dimension");
     auto make = [&](int RU) {
         SyGrid g{};
         g.n = (int)n;
@@ -627,22 +661,28 @@ int launch_kmvm_sym(krr_ctx* ctx, const unsigned char* FA, const unsigned char* 
     const int nbmax = (int)ceil_div(np, SY_PAD);
     float *Vp, *bmax;
     double* vscale;
-    float2 *rowpart, *colpart;
     KRR_RET(bufT(ctx, "sy_vp", (size_t)np, &Vp));
     KRR_RET(bufT(ctx, "sy_bmax", (size_t)nbmax, &bmax));
     KRR_RET(bufT(ctx, "sy_vsc", 1, &vscale));
-    KRR_RET(bufT(ctx, "sy_row", (size_t)(g.G + g.nblk) * g.rows(), &rowpart));
-    KRR_RET(bufT(ctx, "sy_col", (size_t)g.col_base(g.NU), &colpart));
-    KRR_RET(allow_max_dynamic_smem(ctx, (const void*)fn));
     const long long wlimit = ctx->opts.wait_limit_log2 > 0 ? (1LL << ctx->opts.wait_limit_log2)
                                                            : kWaitLimitDefault;
-    launch_pdl(k_sym_pad, nbmax, SY_PAD, 0, ctx->stream, V, (int)n, np, Vp, bmax);
-    KRR_CHECK_LAUNCH();
     const size_t smem = std::max<size_t>(sym_smem(Kp, BN, RU), 120 * 1024);   // one CTA per SM (TMEM)
-    launch_pdl(fn, g.G, SY_THREADS, smem, ctx->stream, FA, FB, Kp, g, Vp, rowpart, colpart, bmax, nbmax, vscale,
-               err, wlimit, ctx->opts.test_stall_copies);
-    KRR_CHECK_LAUNCH();
-    return launch_sym_reduce(ctx, g, rowpart, colpart, V, beta, ex2_bias_scale(ctx), vscale, Q);
+    bool padded = false;
+    return sym_product(ctx, g, [&](const auto& p, void* row, void* col) -> int {
+        using Grid = std::decay_t<decltype(p)>;
+        const sym_fn<Grid> fn = sym_pick<Grid>(nk);
+        float2 *rowpart = (float2*)row, *colpart = (float2*)col;
+        KRR_RET(allow_max_dynamic_smem(ctx, (const void*)fn));
+        if (!padded) {
+            launch_pdl(k_sym_pad, nbmax, SY_PAD, 0, ctx->stream, V, (int)n, np, Vp, bmax);
+            KRR_CHECK_LAUNCH();
+            padded = true;
+        }
+        launch_pdl(fn, p.G, SY_THREADS, smem, ctx->stream, FA, FB, Kp, p, Vp, rowpart, colpart, bmax, nbmax, vscale, err,
+                   wlimit, ctx->opts.test_stall_copies);
+        KRR_CHECK_LAUNCH();
+        return launch_sym_reduce(ctx, p, rowpart, colpart, V, beta, ex2_bias_scale(ctx), vscale, Q, SyPoints());
+    });
 }
 
 }  // namespace krr
