@@ -429,10 +429,14 @@ constexpr int AP_NQ = 8;   // most right-hand sides per pass over F
 // As many as fit: a pass reads F once whatever its columns, and one block an SM with eight is still
 // ahead of two passes (n = 30000, eight columns, against passes of four with more blocks an SM:
 // k = 3800 0.89 against 1.42 ms, 5000 1.21 against 1.87, 6500 1.70 against 2.65).
-static int apply_columns(krr_ctx* ctx, int ldF, int* nq) {
+// The limits are asked for only past AP_SMEM, which with the static part is safe without leave.
+constexpr int AP_SMEM = 40 * 1024;
+static int apply_columns(krr_ctx* ctx, int ldF, int nrhs, int* nq) {
+    *nq = std::min(AP_NQ, nrhs);
+    if (4LL * ldF * *nq <= AP_SMEM) return KRR_OK;
     int optin = 0;
     KRR_TRY_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
-    *nq = std::max(1, std::min(AP_NQ, (optin - 2048) / (4 * ldF)));
+    *nq = std::max(1, std::min(*nq, (optin - 2048) / (4 * ldF)));
     return KRR_OK;
 }
 
@@ -448,8 +452,7 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
     float2* upart;
     double *u, *u1, *v;
     int mq;
-    KRR_RET(apply_columns(ctx, ldF, &mq));
-    mq = std::min(mq, nrhs);
+    KRR_RET(apply_columns(ctx, ldF, nrhs, &mq));
     KRR_RET(bufT(ctx, "ap_upart2", (size_t)nt * mq * ldF, &upart));
     KRR_RET(bufT(ctx, "ap_u", (size_t)mq * k, &u));
     KRR_RET(bufT(ctx, "ap_u1", (size_t)mq * k, &u1));
@@ -476,8 +479,8 @@ int launch_apply_precond(krr_ctx* ctx, const float* R, int nrhs, float* Z, doubl
         KRR_RET(launch_tri_gemv(ctx, ctx->T2, k, u, nq, true, u1));
         KRR_RET(launch_tri_gemv(ctx, ctx->T2t, k, u1, nq, false, v));
         const size_t smem = sizeof(float4) * nq * (ldF / 4);
-        // always: the 48 KB that need no leave are for the dynamic and the kernel's static memory together
-        KRR_RET(allow_max_dynamic_smem(ctx, (const void*)gn));
+        // not only above 48 KB: these are for the dynamic and the kernel's static memory together
+        if (smem > AP_SMEM) KRR_RET(allow_max_dynamic_smem(ctx, (const void*)gn));
         launch_pdl_if(nb < 4 * ctx->num_sms, gn, nb, VT, smem, ctx->stream, ctx->F, n, k, ldF, v, Rq, n, inv_beta, Zq,
                    rz_part ? rz_part + (size_t)q0 * nb : nullptr, rz_part && with_beta ? ctx->cg : nullptr, q0);
         KRR_CHECK_LAUNCH();
