@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <thread>
 #include <vector>
 
 namespace krr {
@@ -389,10 +390,16 @@ int krr_create(krr_ctx** out, const krr_opts* opts, void* stream) {
         delete ctx;
         return KRR_E_CUDA;
     }
+    unsigned flags = 0;
+    if (cudaGetDeviceFlags(&flags) == cudaSuccess)
+        ctx->block = (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
+    else
+        cudaGetLastError();
     if (cudaMalloc(&ctx->cg, sizeof(CGScalars)) != cudaSuccess ||
         cudaMallocHost(&ctx->cg_host, sizeof(CGScalars)) != cudaSuccess ||
         cudaMemsetAsync(ctx->cg, 0, sizeof(CGScalars), ctx->stream) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->cg_read, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&ctx->cg_read, cudaEventDisableTiming |
+                                                    (ctx->block ? cudaEventBlockingSync : 0)) != cudaSuccess) {
         cudaGetLastError();
         if (ctx->cg) cudaFree(ctx->cg);
         if (ctx->cg_host) cudaFreeHost(ctx->cg_host);
@@ -755,11 +762,16 @@ static int square_product64(krr_ctx* ctx, const double* p64, int nrhs, float* ps
 }
 
 // Until the scalar mirror shows the last update of x and r queued; the stream's state is asked now and
-// then, so that an error in what was queued ends the wait.
+// then, so that an error in what was queued ends the wait.  Where the device's waits are to block, an
+// event behind the update is waited for instead, as a stream synchronization would (two queue entries
+// more an iteration); elsewhere the core is offered to other threads every few tens of us.
 static int wait_mirror(krr_ctx* ctx) {
+    if (ctx->block) KRR_TRY_CUDA(cudaEventSynchronize(ctx->cg_read));
     const unsigned long long* seq = &ctx->cg_host->seq;
     auto there = [&]() { return __atomic_load_n(seq, __ATOMIC_ACQUIRE) == ctx->cg_seq; };
     for (unsigned i = 1; !there(); ++i) {
+        if (i & 0xfffu) continue;
+        std::this_thread::yield();
         if (i & 0xffffu) continue;
         const cudaError_t e = cudaStreamQuery(ctx->stream);
         if (e == cudaErrorNotReady) {
@@ -1010,8 +1022,8 @@ int krr_solve(krr_ctx* ctx, const float* X, const float* Y, int nrhs, double tol
                     if (form == 1)
                         KRR_TRY_CUDA(cudaMemcpyAsync(tc_err_host, tc_err_dev, sizeof(int),
                                                      cudaMemcpyDeviceToHost, ctx->stream));
-                    KRR_TRY_CUDA(cudaEventRecord(ctx->cg_read, ctx->stream));
                 }
+                if (hp || ctx->block) KRR_TRY_CUDA(cudaEventRecord(ctx->cg_read, ctx->stream));
                 // The apply of this residual is queued before the host waits for the scalars: the GPU
                 // works while the host decides, and in all but the few iterations that replace the
                 // residual the apply is the one that is needed.

@@ -129,7 +129,8 @@ struct krr_ctx {
     unsigned long long cg_seq = 0;       // updates of x and r that were to write the mirror
     bool want_pq = false;                // a solve's product p -> q: its reduction may form p . q and the step
     bool have_pq = false;                // and did
-    cudaEvent_t cg_read = nullptr;       // the mirror has been copied (FP64 recurrence)
+    cudaEvent_t cg_read = nullptr;       // the scalars of an iteration are on the host, where an event says so
+    bool block = false;                  // host waits give up the core (cudaDeviceScheduleBlockingSync)
 
     // ---- phase timers (off unless krr_profile_enable)
     bool prof = false;
