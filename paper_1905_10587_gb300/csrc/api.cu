@@ -406,6 +406,7 @@ int krr_create(krr_ctx** out, const krr_opts* opts, void* stream) {
         delete ctx;
         return KRR_E_NOMEM;
     }
+    std::memset(ctx->cg_host, 0, sizeof(CGScalars));   // a first wait must not meet its number by chance
     *out = ctx;
     return KRR_OK;
 }
