@@ -66,11 +66,13 @@ k_potf2(double* __restrict__ A, int k, int j0, int nb, double tau, int* __restri
     pdl_entry();
     __shared__ double s[NB][NB + 1], ei[NB][NB + 1], w[NB], sd[NB];
     const int c = threadIdx.x, y = threadIdx.y;
+    const int refused = *info;                     // in a block before: the trailing part was not updated
 #pragma unroll
     for (int r = y; r < NB; r += PF_Y) {
         s[r][c] = (r < nb && c < nb) ? A[(size_t)(j0 + r) * k + j0 + c] : (r == c ? 1.0 : 0.0);
         ei[r][c] = r == c ? 1.0 : 0.0;
     }
+    if (refused) return;                           // one kernel writes it at a time: every thread read the same
     __syncthreads();
     for (int m = 0; m < nb; ++m) {
         const double piv = s[m][m];
@@ -110,8 +112,10 @@ k_potf2(double* __restrict__ A, int k, int j0, int nb, double tau, int* __restri
 // ---- rows i >= j0 + nb: A[i, j0 : j0 + nb] <- A[i, j0 : j0 + nb] L_jj^{-T}, one output a thread
 // (a warp per row: its inputs are read by the warp before any of its outputs is written)
 __global__ void __launch_bounds__(128)
-k_potrf_panel(double* __restrict__ A, int k, int j0, int nb, const double* __restrict__ Linv) {
+k_potrf_panel(double* __restrict__ A, int k, int j0, int nb, const double* __restrict__ Linv,
+              const int* __restrict__ info) {
     pdl_entry();
+    const int refused = *info;                     // a pivot before: no inverse was written
     __shared__ double L[NB][NB + 1];
     __shared__ double x[4][NB];
     for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) L[e / NB][e % NB] = Linv[e];
@@ -119,7 +123,7 @@ k_potrf_panel(double* __restrict__ A, int k, int j0, int nb, const double* __res
     const int i = j0 + nb + blockIdx.x * 4 + wr;
     x[wr][c] = (i < k && c < nb) ? A[(size_t)i * k + j0 + c] : 0.0;
     __syncthreads();
-    if (i >= k || c >= nb) return;
+    if (i >= k || c >= nb || refused) return;
     double v0 = 0.0, v1 = 0.0;
     for (int m = 0; m <= c; m += 2) {              // Linv[c][m] is 0 beyond m = c
         v0 = fma(x[wr][m], L[c][m], v0);
@@ -131,8 +135,9 @@ k_potrf_panel(double* __restrict__ A, int k, int j0, int nb, const double* __res
 // ---- trailing update: A[i, j] -= sum_m A[i, j0+m] A[j, j0+m]  for 16 x 16 tiles (bi >= bj) past j0+nb
 constexpr int DT = 16;
 __global__ void __launch_bounds__(DT * DT)
-k_potrf_update(double* __restrict__ A, int k, int j0, int nb, int t0) {
+k_potrf_update(double* __restrict__ A, int k, int j0, int nb, int t0, const int* __restrict__ info) {
     pdl_entry();
+    const int refused = *info;
     // blockIdx.x enumerates the lower-triangular tile pairs of the trailing matrix
     const int p = blockIdx.x;
     int bi = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
@@ -150,7 +155,7 @@ k_potrf_update(double* __restrict__ A, int k, int j0, int nb, int t0) {
     __syncthreads();
     const int c = threadIdx.x % DT, r = threadIdx.x / DT;
     const int gi = r0 + r, gj = c0 + c;
-    if (gi >= k || gj >= k || gj > gi) return;
+    if (gi >= k || gj >= k || gj > gi || refused) return;
     double v0 = 0.0, v1 = 0.0;
 #pragma unroll
     for (int m = 0; m < NB; m += 2) {
@@ -181,10 +186,11 @@ int launch_potrf(krr_ctx* ctx, double* A, int k, int* info_host, double* dinv, d
         KRR_CHECK_LAUNCH();
         const int rest = k - j0 - nb;
         if (rest <= 0) break;
-        launch_pdl(k_potrf_panel, ceil_div(rest, 4), 128, 0, ctx->stream, A, k, j0, nb, Lj);
+        launch_pdl(k_potrf_panel, ceil_div(rest, 4), 128, 0, ctx->stream, A, k, j0, nb, Lj, info);
         KRR_CHECK_LAUNCH();
         const int tb = (rest + DT - 1) / DT;
-        launch_pdl(k_potrf_update, tb * (tb + 1) / 2, DT * DT, 0, ctx->stream, A, k, j0, nb, j0 + nb);
+        launch_pdl(k_potrf_update, tb * (tb + 1) / 2, DT * DT, 0, ctx->stream, A, k, j0, nb, j0 + nb,
+                   info);
         KRR_CHECK_LAUNCH();
     }
     k_zero_upper<<<ceil_div((long long)k * k, 256), 256, 0, ctx->stream>>>(A, k);

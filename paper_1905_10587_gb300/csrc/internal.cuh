@@ -405,8 +405,8 @@ int launch_strong_rrqr(krr_ctx* ctx, float* Y, long long n, int l, int ldy, int 
 // dense64.cu
 int launch_kss(krr_ctx* ctx, const float* XS, int k, int d, double sigma, double* A);
 // In-place lower Cholesky of the k x k row-major A (upper part ignored).  Sets *info
-// (host) to 0 or to 1 + the first column whose pivot is <= tau (or not finite); the
-// columns before it are final.
+// (host) to 0 or to 1 + the first column whose pivot is <= tau (or not finite); then only
+// the 32-column blocks before that column's own are final, and so are their inverses.
 // dinv (potrf_dinv) receives the inverses of L's diagonal blocks, for launch_tri_inverse.
 int potrf_dinv(krr_ctx* ctx, int k, double** dinv);
 int launch_potrf(krr_ctx* ctx, double* A, int k, int* info, double* dinv, double tau = 0.0);
