@@ -224,8 +224,8 @@ k_rect_ff(const float* __restrict__ Xr, int nr, const float2* __restrict__ NR_, 
 // groups; a thread holds R rows and takes one column at a time.  Sums are float-float over one
 // column tile (rows) or over R rows, 8 lanes (columns), and FP64 beyond, as above.
 // R = 4, 2 or 1: units of 256 x 128, 128 x 128 or 64 x 64 pairs, so that small sets fill the chip.
-// Measured (one residual, against k_rect_ff): n = 30011, d = 8 2.90 ms against 5.00 (68% of the FMA
-// pipe's rate for the operations above), n = 10^5 30.9 against 55 ms.
+// Measured (one residual, against k_rect_ff): n = 30011, d = 8 2.90 ms against 5.00 (71% of the FMA
+// pipe's rate, 2.06 ms for the operations above), n = 10^5 30.9 against 55 ms.
 template <int R>
 constexpr int sff_bn() { return R == 1 ? 64 : 128; }
 constexpr int SFF_T = 256, SFF_NW = SFF_T / 32;

@@ -24,14 +24,15 @@
 // Split.  The (block, unit) pairs of all row blocks form one sequence, cut into one equal run per
 // SM: no tail wave, and a run touches few row blocks.  Column sums leave as float-float pairs in
 // slot I of their column unit, row sums in one slot per (run, row block); k_sym_reduce adds the
-// slots of every point in a fixed order, so results do not depend on timing.
+// slots of every point in a fixed order, so results do not depend on timing.  Large sets take their row
+// blocks in panels (SyPanel), a launch each.
 //
-// Measured, n = 10^5, d = 8, the whole krr_kmvm call (about 0.21 ms of it packs points and
-// features): 1.149 ms, against 1.754 ms for k_kmvm_tc; n = 2048 0.114 against 0.131 ms, and ahead at
-// every n down to 200, so it takes every square product with one right-hand side.  A solve of
-// that size (785 products) went from 1.69 to 1.21 s.  The kernel keeps the MUFU 59% busy; what is left
-// is issue: 437 instructions per warp and tile of which 256 are ex2 and FMA, with two warps per
-// scheduler.  Sixteen epilogue warps (64 columns each) measured 5% slower, two warp groups on alternate
+// Measured, n = 10^5, d = 8, the whole krr_kmvm call (about 0.09 ms of it packs points and features and
+// adds the slots): 1.00 ms; 1.149 against 1.754 ms for k_kmvm_tc when both still took 0.21 ms to pack,
+// n = 2048 0.114 against 0.131 ms then, and ahead at every n down to 200, so it takes every square
+// product with one right-hand side.  The kernel keeps the MUFU 53 to 55% busy and issues in 56% of the
+// cycles; the largest stall is fixed-latency dependences, with two warps per scheduler (437
+// instructions per warp and tile, of which 256 are ex2 and FMA).  Sixteen epilogue warps (64 columns each) measured 5% slower, two warp groups on alternate
 // tiles 10% slower.  Fetching v a tile ahead and asking for the next tile's barrier a step ahead
 // gave 5% together, folding row and column sums under the next tile's exponentials 4%.
 #include "internal.cuh"
